@@ -18,6 +18,7 @@ namespace shl {
 
 constexpr int kSlice = 32;          // SELL slice height (one warp)
 constexpr int kBlock = 256;         // threads of every CTA of the persistent solve kernel
+constexpr int kMaxAmgLevels = 12;   // multigrid levels of one instance (build_amg's limit)
 constexpr int kForceBlock = 128;    // threads of a force tile
 constexpr int kMaxTeamWaitMs = 4000;  // default bound of a team-barrier wait (Sched::wait_ns)
 constexpr int kBarWords = 64;       // barrier words per team (256 bytes): a 64-bit arrival counter at [0, 2),
