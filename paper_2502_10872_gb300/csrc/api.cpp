@@ -910,6 +910,7 @@ int setup_amg(shell_handle *h, const HostTopo &T, int mode, bool stage, const st
       D.n = n;
       D.n_next = (l < L - 1) ? H.levels[l + 1].A.n : 0;
       D.omega = H.levels[l].omega;
+      D.omega32 = float(D.omega);
       if (l > 0) {
         D.a_ptr = C.take<int32_t>(As[l].sl_ptr.size());
         D.a_col = C.take<int32_t>(As[l].sl_col.size());

@@ -78,6 +78,7 @@ struct AmgDev {
   float *r_val32;
   double *r_val64;
   double omega;                  // damped-Jacobi weight
+  float omega32, pad;            // the same, rounded
   void *b, *x, *r, *y;           // right-hand side, pre-smoothed x, its residual, cycle output (AoS)
   HaloDev ha, hp, hr;            // gather lists of A, Ps and Rs (FP32 products)
 };

@@ -208,7 +208,9 @@ __device__ void stage_chunk(ChunkStage &cs, const Inst &I, const Team &tm, int c
 
 // sum all chunk partials of an instance in a fixed order; result broadcast to the CTA. Flips the bank, so
 // the next phase may write partials while slower CTAs of the team still read these.
-__device__ void team_reduce(const Inst &I, Team &tm, double out[3]) {
+// then(sum): run by the thread that holds the sums, before they are broadcast.
+template <typename F>
+__device__ __forceinline__ void team_reduce(const Inst &I, Team &tm, double out[3], F then) {
   __shared__ double res[3];
   const double *part = I.part + 4 * (size_t)tm.bank * I.n_chunks;
   const int n_chunks = I.n_chunks;
@@ -227,12 +229,16 @@ __device__ void team_reduce(const Inst &I, Team &tm, double out[3]) {
       res[0] = a0;
       res[1] = a1;
       res[2] = a2;
+      then(res);
     }
   }
   __syncthreads();
   out[0] = res[0];
   out[1] = res[1];
   out[2] = res[2];
+}
+__device__ void team_reduce(const Inst &I, Team &tm, double out[3]) {
+  team_reduce(I, tm, out, [](const double *) {});
 }
 
 // ------------------------------------------------------------------ precision traits
@@ -552,6 +558,30 @@ __device__ __noinline__ void tangent_corr(const Inst &I, const G *u, int row, R 
   cz = dt2 * y.z;
 }
 
+// ------------------------------------------------------------------ level views
+template <typename R>
+struct LevelVal;
+template <>
+struct LevelVal<float> {
+  __device__ static const float *a(const AmgDev &L) { return L.a_val32; }
+  __device__ static const float *p(const AmgDev &L) { return L.p_val32; }
+  __device__ static const float *r(const AmgDev &L) { return L.r_val32; }
+  __device__ static const float *dinv(const AmgDev &L) { return L.dinv32; }
+  __device__ static const float *cinv(const Inst &I) { return I.amg_cinv32; }
+  __device__ static const float *dense(const Inst &I) { return I.amg_dense32; }
+  __device__ static float omega(const AmgDev &L) { return L.omega32; }
+};
+template <>
+struct LevelVal<double> {
+  __device__ static const double *a(const AmgDev &L) { return L.a_val64; }
+  __device__ static const double *p(const AmgDev &L) { return L.p_val64; }
+  __device__ static const double *r(const AmgDev &L) { return L.r_val64; }
+  __device__ static const double *dinv(const AmgDev &L) { return L.dinv64; }
+  __device__ static const double *cinv(const Inst &I) { return I.amg_cinv64; }
+  __device__ static const double *dense(const Inst &I) { return I.amg_dense64; }
+  __device__ static double omega(const AmgDev &L) { return L.omega; }
+};
+
 // ------------------------------------------------------------------ phases
 // Per-stencil forces of the instance at the positions of this launch (x, or the chord iterate xk of exact
 // backward Euler), in the instance's precision, written to its contribution slots (one writer per slot). The
@@ -668,7 +698,7 @@ __device__ void phase_resid(const Inst &I, const Team &tm) {
   const bool amg = I.amg_levels > 0;
   typename Vec<R>::G *b0 = amg ? reinterpret_cast<typename Vec<R>::G *>(I.amg[0].b) : nullptr;
   typename Vec<R>::G *x0 = amg ? reinterpret_cast<typename Vec<R>::G *>(I.amg[0].x) : nullptr;
-  const R om0 = amg ? R(I.amg[0].omega) : R(0);
+  const R om0 = amg ? LevelVal<R>::omega(I.amg[0]) : R(0);
   const D4 *g64 = reinterpret_cast<const D4 *>(I.g64);
   R *r = reinterpret_cast<R *>(I.r);
   double *xs = reinterpret_cast<double *>(I.xs);
@@ -817,7 +847,7 @@ __device__ void phase_update(const Inst &I, const Team &tm, R alpha, R beta, boo
   // row-local, so it is done here from the new r
   typename Vec<R>::G *b0 = amg ? reinterpret_cast<typename Vec<R>::G *>(I.amg[0].b) : nullptr;
   typename Vec<R>::G *x0 = amg ? reinterpret_cast<typename Vec<R>::G *>(I.amg[0].x) : nullptr;
-  const R om0 = amg ? R(I.amg[0].omega) : R(0);
+  const R om0 = amg ? LevelVal<R>::omega(I.amg[0]) : R(0);
   ROWS_BEGIN(I, tm)
   const R di = dinv[row];
   R uo[3];
@@ -854,27 +884,6 @@ __device__ void phase_update(const Inst &I, const Team &tm, R alpha, R beta, boo
 
 // ------------------------------------------------------------------ multigrid V-cycle (preconditioner)
 // SpMV helpers on one level's arrays (SELL-32: the folded prolongation Ps, and the level-0 operator).
-template <typename R>
-struct LevelVal;
-template <>
-struct LevelVal<float> {
-  __device__ static const float *a(const AmgDev &L) { return L.a_val32; }
-  __device__ static const float *p(const AmgDev &L) { return L.p_val32; }
-  __device__ static const float *r(const AmgDev &L) { return L.r_val32; }
-  __device__ static const float *dinv(const AmgDev &L) { return L.dinv32; }
-  __device__ static const float *cinv(const Inst &I) { return I.amg_cinv32; }
-  __device__ static const float *dense(const Inst &I) { return I.amg_dense32; }
-};
-template <>
-struct LevelVal<double> {
-  __device__ static const double *a(const AmgDev &L) { return L.a_val64; }
-  __device__ static const double *p(const AmgDev &L) { return L.p_val64; }
-  __device__ static const double *r(const AmgDev &L) { return L.r_val64; }
-  __device__ static const double *dinv(const AmgDev &L) { return L.dinv64; }
-  __device__ static const double *cinv(const Inst &I) { return I.amg_cinv64; }
-  __device__ static const double *dense(const Inst &I) { return I.amg_dense64; }
-};
-
 // plain y_i = sum_j m_ij v_j over a SELL-32 matrix (the folded prolongation Ps; the level-0 operator in FP64)
 template <typename R, typename G>
 __device__ inline void sell_plain(const int32_t *sp, const int32_t *sc, const R *sv, const G *v, int row, R &ax,
@@ -996,7 +1005,7 @@ __device__ __forceinline__ void restrict_blk(const AmgDev &A, const AmgDev &C, b
   G *xc = reinterpret_cast<G *>(C.x);
   const R *dinvc = LevelVal<R>::dinv(C);
   const R *val = LevelVal<R>::r(A);
-  const R omc = R(C.omega);
+  const R omc = LevelVal<R>::omega(C);
   const int n = A.n_next;
   const int lane = threadIdx.x & 31;
   const int row = blk * kRows + (int)(threadIdx.x >> 2);
@@ -1068,7 +1077,7 @@ __device__ void lv_up(const AmgDev &A, const AmgDev &C, typename Vec<R>::G *y, c
   const G *rr = reinterpret_cast<const G *>(A.r);
   const G *yc = reinterpret_cast<const G *>(C.y);
   const R *dinv = LevelVal<R>::dinv(A);
-  const R om = R(A.omega);
+  const R om = LevelVal<R>::omega(A);
   for (int ch = tm.rank; ch * kBlock < A.n; ch += tm.size) {
     const int row = ch * kBlock + (int)threadIdx.x;
     R ax, ay, az;
@@ -1206,7 +1215,7 @@ __device__ void lv_smooth4(const AmgDev &A, const typename Vec<R>::G *x, typenam
   typedef typename Vec<R>::G G;
   const G *b = reinterpret_cast<const G *>(A.b);
   const R *dinv = LevelVal<R>::dinv(A);
-  const R om = R(A.omega);
+  const R om = LevelVal<R>::omega(A);
   for (int ch = tm.rank; ch * (kBlock / 4) < A.n; ch += tm.size) {
     const int row = ch * (kBlock / 4) + (int)(threadIdx.x >> 2);
     const bool valid = row < A.n;
@@ -1288,7 +1297,7 @@ __device__ bool coarsest(const Inst &I, const Team &tm) {
   }
   G *x = reinterpret_cast<G *>(C.x);
   const R *dinv = LevelVal<R>::dinv(C);
-  const R om = R(C.omega);
+  const R om = LevelVal<R>::omega(C);
   LEVEL_ROWS_BEGIN(C.n, tm)
   const G bi = ldg4(b + row);
   const R d = om * dinv[row];
@@ -1401,42 +1410,72 @@ __device__ bool vcycle(const Inst &I, const Team &tm) {
   return true;
 }
 
+// Scalars of the recurrence, computed by one thread of the CTA from the reduced sums and read by the others from
+// shared memory: three dependent FP64 divisions in every thread occupied the FP64 pipe (2 operations per clock and
+// SM on GB300) for several thousand clocks of each iteration. Per call, with the smoother's weight read in FP32
+// instead of converted by every thread in every phase: 512 x 512 plate 19.0 -> 18.2 ms (4 steps), 128 x 128 cylinder
+// 5.91 -> 5.79 ms (8 steps), FP64 7.97 -> 7.83 ms (4 steps), batch of 256 36.7 -> 36.4 ms (8 steps).
+struct CgScalars {
+  double alpha, beta, gamma, rho;
+  float alpha32, beta32;
+  int verdict;   // 1: go on, 0: converged, -1: iteration cap, -3: not finite
+};
+__device__ inline CgScalars &cg_state() {
+  __shared__ CgScalars s;
+  return s;
+}
+template <typename R>
+struct CgCoef;
+template <>
+struct CgCoef<float> {
+  __device__ static float alpha(const CgScalars &s) { return s.alpha32; }
+  __device__ static float beta(const CgScalars &s) { return s.beta32; }
+};
+template <>
+struct CgCoef<double> {
+  __device__ static double alpha(const CgScalars &s) { return s.alpha; }
+  __device__ static double beta(const CgScalars &s) { return s.beta; }
+};
+template <typename R>
+__device__ inline void cg_scalars(const double *sum, int it, double tol2, int max_it) {
+  CgScalars &s = cg_state();
+  const double gn = sum[0], dn = sum[1], rho = sum[2];
+  s.rho = rho;
+  if (!isfinite(rho) || !isfinite(gn) || !isfinite(dn)) {
+    s.verdict = -3;
+  } else if (rho <= tol2) {
+    s.verdict = 0;
+  } else if (it >= max_it) {
+    s.verdict = -1;
+  } else {
+    const double bn = it == 0 ? 0.0 : gn / s.gamma;
+    s.alpha = it == 0 ? gn / dn : gn / (dn - bn * gn / s.alpha);
+    s.beta = bn;
+    s.gamma = gn;
+    s.alpha32 = float(s.alpha);
+    s.beta32 = float(bn);
+    s.verdict = 1;
+  }
+}
+
 // Chronopoulos-Gear PCG iterations on A x = r0, given r (initial residual), x (initial guess) and
 // g = D^-1 r. Stops when (r,r) <= tol2 (absolute). Returns iterations (>= 0), -1 on cap, -2 on abort,
 // -3 on a non-finite reduction.
 template <typename R, bool NT>
 __device__ int cg_loop(const Inst &I, Team &tm, double *x, double tol2, int max_it, double *rho_out) {
   if (!team_sync(tm)) return -2;
-  if (I.amg_levels > 0 && !vcycle<R, NT>(I, tm)) return -2;
-  phase_spmv<R, NT>(I, tm);
-  if (!team_sync(tm)) return -2;
-  double red[3];
-  team_reduce(I, tm, red);
-  double gamma = red[0], delta = red[1], rho = red[2];
-  *rho_out = rho;
-  if (!isfinite(rho) || !isfinite(gamma) || !isfinite(delta)) return -3;
-  if (rho <= tol2) return 0;
-  double alpha = gamma / delta, beta = 0.0;
-  bool first = true;
-  for (int it = 1; it <= max_it; ++it) {
-    phase_update<R>(I, tm, R(alpha), R(beta), first, x, alpha);
-    if (!team_sync(tm)) return -2;
+  for (int it = 0;; ++it) {
     if (I.amg_levels > 0 && !vcycle<R, NT>(I, tm)) return -2;
     phase_spmv<R, NT>(I, tm);
     if (!team_sync(tm)) return -2;
-    team_reduce(I, tm, red);
-    const double gn = red[0], dn = red[1];
-    rho = red[2];
-    *rho_out = rho;
-    if (!isfinite(rho) || !isfinite(gn) || !isfinite(dn)) return -3;
-    if (rho <= tol2) return it;
-    const double bn = gn / gamma;
-    alpha = gn / (dn - bn * gn / alpha);
-    beta = bn;
-    gamma = gn;
-    first = false;
+    double red[3];
+    team_reduce(I, tm, red, [&](const double *sum) { cg_scalars<R>(sum, it, tol2, max_it); });
+    const CgScalars &S = cg_state();
+    *rho_out = S.rho;
+    if (S.verdict <= 0) return S.verdict == 0 ? it : S.verdict;
+    phase_update<R>(I, tm, CgCoef<R>::alpha(S), CgCoef<R>::beta(S), it == 0, x, S.alpha);
+    if (!team_sync(tm)) return -2;
   }
-  return -1;
 }
 
 // sol += xs (the inner correction, accumulated in FP64); g64 = sol
@@ -1713,6 +1752,7 @@ __device__ bool solve_fp32r(const Inst &I, Team &tm) {
   }
   int total = 0, rounds = 0;
   double rel = 0.0, ref = bb;
+  const bool writer = tm.rank == 0 && threadIdx.x == 0;   // the thread that reports rel (see cg_scalars on the others)
   bool early = false;
   if (bb > 0.0) {
     double tol_ref2 = I.refine_rtol * I.refine_rtol * bb;
@@ -1737,7 +1777,7 @@ __device__ bool solve_fp32r(const Inst &I, Team &tm) {
         // no need to solve below a tenth of the nonlinear target (inexact Newton)
         tol_ref2 = fmax(I.refine_rtol * I.refine_rtol * r2, k > 0 ? nl_floor2(I) : 0.0);
       }
-      rel = sqrt(r2 / ref);
+      if (writer) rel = sqrt(r2 / ref);
       if (r2 <= tol_ref2) break;
       if (rounds >= I.refine_max) {
         set_status(I, tm, SHELL_ERR_NOT_CONVERGED, total, rounds, rel);
@@ -1883,7 +1923,7 @@ static SolveFn solve_fn(int prec, int occ) {
 int solve_halo_cap(int prec, int occ) {
   if (prec == 1) return 0;
   if (prec == 2 && occ >= 5) return 2048;
-  if (prec == 2 && occ == 4) return 3072;
+  if (prec == 2 && occ == 4) return 2880;
   return 4096;
 }
 
