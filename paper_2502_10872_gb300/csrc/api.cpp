@@ -187,11 +187,10 @@ namespace {
 
 // Device properties queried once (atomics: handles may be created on several threads; racing threads
 // compute the same value).
-// CTAs per SM of the solve variant compiled for `occ` (FP32: variants for 3, 4, 5; others one variant)
+// CTAs per SM of the solve variant compiled for `occ` (FP32: variants for 2, 3, 4; others one variant)
 int blocks_per_sm_cached(int prec, int occ = 3) {
-  static std::atomic<int> n[4][6] = {{-1, -1, -1, -1, -1, -1}, {-1, -1, -1, -1, -1, -1}, {-1, -1, -1, -1, -1, -1},
-                                     {-1, -1, -1, -1, -1, -1}};
-  occ = std::max(1, std::min(5, occ));
+  static std::atomic<int> n[4][5] = {{-1, -1, -1, -1, -1}, {-1, -1, -1, -1, -1}, {-1, -1, -1, -1, -1}, {-1, -1, -1, -1, -1}};
+  occ = std::max(1, std::min(4, occ));
   int v = n[prec][occ].load();
   if (v < 0) {
     v = std::max(1, solve_blocks_per_sm(prec, occ));
@@ -199,7 +198,7 @@ int blocks_per_sm_cached(int prec, int occ = 3) {
   }
   return v;
 }
-int max_occ(int prec) { return prec == 2 ? blocks_per_sm_cached(2, 5) : blocks_per_sm_cached(prec, 2); }
+int max_occ(int prec) { return prec == 2 ? blocks_per_sm_cached(2, 4) : blocks_per_sm_cached(prec, 2); }
 int max_clusters_cached(int prec) {
   static std::atomic<int> n[4] = {-1, -1, -1, -1};
   int v = n[prec].load();
@@ -1750,10 +1749,9 @@ int shell_batch_autotune(shell_batch *b, int32_t steps_per_trial, double *out_ms
   if (b->n_active == 0) return SHELL_OK;
   const int occ_max = max_occ(b->prec);
   int occs[3] = {1, std::max(1, occ_max / 2), occ_max};
-  if (b->prec == 2) {   // the FP32 variants compiled for 3, 4 and 5 CTAs per SM
+  if (b->prec == 2) {   // the FP32 variants compiled for 3 and 4 CTAs per SM
     occs[0] = blocks_per_sm_cached(2, 3);
-    occs[1] = blocks_per_sm_cached(2, 4);
-    occs[2] = blocks_per_sm_cached(2, 5);
+    occs[1] = occs[2] = blocks_per_sm_cached(2, 4);
   }
   const double scales[3] = {0.5, 1.0, 2.0};
   double best = 1e300;

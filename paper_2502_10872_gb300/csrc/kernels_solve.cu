@@ -49,11 +49,6 @@ __device__ inline unsigned long long gtimer() {
   asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
   return t;
 }
-__device__ inline unsigned int ld_acquire(const unsigned int *p) {
-  unsigned int v;
-  asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
-  return v;
-}
 __device__ inline int ld_volatile_i(const int *p) { return *((volatile const int *)p); }
 
 struct Team {
@@ -83,36 +78,35 @@ __device__ inline double *part_of(const Inst &I, const Team &tm, int ch) {
   return I.part + 4 * ((size_t)tm.bank * I.n_chunks + ch);
 }
 
-__device__ inline unsigned long long ld_acquire64(const unsigned long long *p) {
-  unsigned long long v;
-  asm volatile("ld.acquire.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
-  return v;
-}
-
 // Bounded global-memory barrier among `parties` arrivals on the team's words (thread 0 of the caller only).
 // The team's 64-bit arrival counter only grows: it is zeroed when the team layout is built (and after an
 // abandoned launch), and every CTA of a team passes the same barriers, so an episode starts at a multiple
 // of `parties` and ends when the counter reaches the next one. The last arrival's own increment releases the
 // others (no reset or generation word to write after it), and no word is read before arriving.
 // Returns 0 if it gave up (timeout, or abort raised elsewhere).
+// One acquire-release increment and one acquire fence after relaxed polls (152 CTAs: 1.25 us, against 1.4 us with a full
+// fence on each side of a relaxed increment); the abort flag, another L2 round trip, is looked at only every 16th poll.
 __device__ int global_arrive_wait(const Team &tm, unsigned int parties) {
   unsigned long long *count = reinterpret_cast<unsigned long long *>(tm.bar);
-  __threadfence();   // this CTA's writes of the phase are visible before its arrival
-  const unsigned long long o = atomicAdd(count, 1ull);
+  unsigned long long o;
+  // release: this CTA's writes of the phase (ordered before by the CTA barrier) are visible before its arrival
+  asm volatile("atom.add.acq_rel.gpu.global.u64 %0, [%1], 1;" : "=l"(o) : "l"(count) : "memory");
   const unsigned long long target = (o / parties + 1ull) * parties;
   if (o + 1ull != target) {
     const unsigned long long t0 = gtimer();
     const unsigned long long limit = tm.wait_ns;
-    while (ld_acquire64(count) < target) {
-      if (ld_volatile_i(tm.abort_flag)) return 0;
+    for (unsigned int polls = 1;; ++polls) {
+      unsigned long long v;
+      asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(count) : "memory");
+      if (v >= target) break;
+      if (polls % 16 == 0 && ld_volatile_i(tm.abort_flag)) return 0;
       if (gtimer() - t0 > limit) {
         atomicExch(tm.abort_flag, 1);
         return 0;
       }
-      __nanosleep(32);
     }
+    asm volatile("fence.acq_rel.gpu;" ::: "memory");
   }
-  __threadfence();
   return 1;
 }
 
@@ -212,12 +206,17 @@ __device__ void stage_chunk(ChunkStage &cs, const Inst &I, const Team &tm, int c
 template <typename F>
 __device__ __forceinline__ void team_reduce(const Inst &I, Team &tm, double out[3], F then) {
   __shared__ double res[3];
+  __shared__ double wsum[kBlock / 32][3];
   const double *part = I.part + 4 * (size_t)tm.bank * I.n_chunks;
   const int n_chunks = I.n_chunks;
-  tm.bank ^= 1;
-  if (threadIdx.x < 32) {
-    double a0 = 0.0, a1 = 0.0, a2 = 0.0;
-    for (int c = threadIdx.x; c < n_chunks; c += 32) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  // every thread takes the chunks c, c + 256, ...; the threads of a warp are added by a tree, then the warps (one warp
+  // alone takes up to 32 chunks). One warp summing all 1,024 chunks of the 512 x 512 plate spent 16 us per reduction on 32
+  // dependent rounds of L2 loads.
+  const bool wide = n_chunks > 32;
+  double a0 = 0.0, a1 = 0.0, a2 = 0.0;
+  if (wide || warp == 0) {
+    for (int c = threadIdx.x; c < n_chunks; c += kBlock) {
       a0 += __ldcg(part + 4 * c);
       a1 += __ldcg(part + 4 * c + 1);
       a2 += __ldcg(part + 4 * c + 2);
@@ -225,12 +224,33 @@ __device__ __forceinline__ void team_reduce(const Inst &I, Team &tm, double out[
     a0 = warp_sum(a0);
     a1 = warp_sum(a1);
     a2 = warp_sum(a2);
-    if (threadIdx.x == 0) {
-      res[0] = a0;
-      res[1] = a1;
-      res[2] = a2;
-      then(res);
+  }
+  if (wide) {
+    if (lane == 0) {
+      wsum[warp][0] = a0;
+      wsum[warp][1] = a1;
+      wsum[warp][2] = a2;
     }
+    __syncthreads();
+    if (warp == 0) {
+      const bool in = lane < kBlock / 32;
+      a0 = in ? wsum[lane][0] : 0.0;
+      a1 = in ? wsum[lane][1] : 0.0;
+      a2 = in ? wsum[lane][2] : 0.0;
+#pragma unroll
+      for (int o = kBlock / 64; o > 0; o >>= 1) {
+        a0 += __shfl_down_sync(0xffffffffu, a0, o);
+        a1 += __shfl_down_sync(0xffffffffu, a1, o);
+        a2 += __shfl_down_sync(0xffffffffu, a2, o);
+      }
+    }
+  }
+  if (threadIdx.x == 0) {
+    res[0] = a0;
+    res[1] = a1;
+    res[2] = a2;
+    tm.bank ^= 1;   // the partials' readers of this CTA have read theirs
+    then(res);
   }
   __syncthreads();
   out[0] = res[0];
@@ -832,6 +852,12 @@ __device__ void phase_spmv(const Inst &I, const Team &tm) {
       R ax, ay, az;
       typename Vec<R>::G u;
       const int row = blk * kBlock + (int)threadIdx.x;
+      R r0 = R(0), r1 = R(0), r2 = R(0);   // loaded before the product, whose latency hides theirs
+      if (row < nv) {
+        r0 = r[row];
+        r1 = r[nv + row];
+        r2 = r[2 * nv + row];
+      }
       if constexpr (sizeof(R) == 4) {
         if (st) {
           staged_row<true>(I.h0, blk, g, I.sl_ptr, val, I.rs32, row, row < nv, ax, ay, az, u);
@@ -864,7 +890,6 @@ __device__ void phase_spmv(const Inst &I, const Team &tm) {
       w[row] = ax;
       w[nv + row] = ay;
       w[2 * nv + row] = az;
-      const R r0 = r[row], r1 = r[nv + row], r2 = r[2 * nv + row];
       gu += r0 * R(u.x) + r1 * R(u.y) + r2 * R(u.z);
       wu += ax * R(u.x) + ay * R(u.y) + az * R(u.z);
       rr2 += r0 * r0 + r1 * r1 + r2 * r2;
@@ -899,25 +924,37 @@ __device__ void phase_update(const Inst &I, const Team &tm, R alpha, R beta, boo
   const R om0 = amg ? LevelVal<R>::omega(I.amg[0]) : R(0);
   ROWS_BEGIN(I, tm)
   const R di = dinv[row];
-  R uo[3];
+  // all loads before the first store: the stores may alias the next component's loads for all the compiler knows
+  R uo[3], ro[3], po[3], so[3], wo[3];
+  double xo[3];
   if (amg) {
     const typename Vec<R>::G gu = ldg4(g + row);
     uo[0] = R(gu.x);
     uo[1] = R(gu.y);
     uo[2] = R(gu.z);
   }
+#pragma unroll
+  for (int c = 0; c < 3; ++c) {
+    const int k = c * nv + row;
+    ro[c] = r[k];
+    wo[c] = w[k];
+    if (!first) {
+      po[c] = p[k];
+      so[c] = s[k];
+    }
+    xo[c] = x[k];
+  }
   R rv[3];
 #pragma unroll
   for (int c = 0; c < 3; ++c) {
     const int k = c * nv + row;
-    const R rc = r[k];
-    const R u = amg ? uo[c] : di * rc;
-    const R pc = first ? u : u + beta * p[k];
-    const R sc = first ? w[k] : w[k] + beta * s[k];
+    const R u = amg ? uo[c] : di * ro[c];
+    const R pc = first ? u : u + beta * po[c];
+    const R sc = first ? wo[c] : wo[c] + beta * so[c];
     p[k] = pc;
     s[k] = sc;
-    x[k] += alpha_x * double(pc);
-    const R rn = rc - alpha * sc;
+    x[k] = xo[c] + alpha_x * double(pc);
+    const R rn = ro[c] - alpha * sc;
     r[k] = rn;
     rv[c] = rn;
   }
@@ -1403,26 +1440,45 @@ __device__ bool dense_level(const Inst &I, const Team &tm) {
   const int r0 = tm.rank * per, r1 = min(n, r0 + per);
   double(*part)[kBlock / 32][3] = stage_buf();   // [32 rows][8 warps][3], free between reductions
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  // b staged in shared memory (FP32) while the first columns are on their way; the next U columns are loaded before
+  // the present ones are used
+  R a[U], an[U];
+  auto columns = [&](R *to, int i, int j0) {
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const int j = j0 + 8 * u;
+      to[u] = (i < r1 && j < n) ? B[(size_t)j * n + i] : R(0);
+    }
+  };
+  columns(a, r0 + lane, w);
+  bool st = false;
+  if constexpr (sizeof(R) == 4) {
+    st = n <= tm.cap;
+    if (st) {
+      for (int j = threadIdx.x; j < n; j += kBlock) sh_halo[j] = b[j];
+      __syncthreads();
+    }
+  }
   for (int base = r0; base < r1; base += 32) {
     const int i = base + lane;
+    if (base != r0) columns(a, i, w);
     R ax = R(0), ay = R(0), az = R(0);
-    if (i < r1) {
-      for (int j0 = w; j0 < n; j0 += 8 * U) {
-        R a[U];
-        G t[U];
+    for (int j0 = w; j0 < n; j0 += 8 * U) {
+      if (j0 + 8 * U < n) columns(an, i, j0 + 8 * U);
 #pragma unroll
-        for (int u = 0; u < U; ++u) {
-          const int j = j0 + 8 * u;
-          a[u] = j < n ? B[(size_t)j * n + i] : R(0);
-          t[u] = ldg4(b + (j < n ? j : 0));
-        }
-#pragma unroll
-        for (int u = 0; u < U; ++u) {
-          ax += a[u] * R(t[u].x);
-          ay += a[u] * R(t[u].y);
-          az += a[u] * R(t[u].z);
-        }
+      for (int u = 0; u < U; ++u) {
+        const int j = j0 + 8 * u < n ? j0 + 8 * u : 0;
+        G t;
+        if constexpr (sizeof(R) == 4)
+          t = st ? sh_halo[j] : b[j];
+        else
+          t = ldg4(b + j);
+        ax += a[u] * R(t.x);
+        ay += a[u] * R(t.y);
+        az += a[u] * R(t.z);
       }
+#pragma unroll
+      for (int u = 0; u < U; ++u) a[u] = an[u];
     }
     part[lane][w][0] = double(ax);
     part[lane][w][1] = double(ay);
@@ -1533,11 +1589,10 @@ __device__ void phase_accumulate(const Inst &I, const Team &tm) {
   const double *xs = reinterpret_cast<const double *>(I.xs);
   ROWS_BEGIN(I, tm)
   double sv[3];
-  for (int c = 0; c < 3; ++c) {
-    const int k = c * nv + row;
-    sv[c] = I.sol[k] + xs[k];
-    I.sol[k] = sv[c];
-  }
+#pragma unroll
+  for (int c = 0; c < 3; ++c) sv[c] = I.sol[c * nv + row] + xs[c * nv + row];   // loads before stores
+#pragma unroll
+  for (int c = 0; c < 3; ++c) I.sol[c * nv + row] = sv[c];
   reinterpret_cast<D4 *>(I.g64)[row] = {sv[0], sv[1], sv[2], 0.0};
   ROWS_END
 }
@@ -1548,14 +1603,24 @@ __device__ void phase_commit(const Inst &I, const Team &tm) {
   const int nv = I.nv;
   const bool st = I.nl_static != 0;
   ROWS_BEGIN(I, tm)
+  double v[3], v0[3], p[3], p2[3], x[3];   // loads before stores
+#pragma unroll
   for (int c = 0; c < 3; ++c) {
     const int k = c * nv + row;
-    const double v = I.sol[k];
-    I.vprev3[k] = st ? 0.0 : I.vprev2[k];
-    I.vprev2[k] = st ? 0.0 : I.vprev[k];
-    I.vprev[k] = st ? 0.0 : I.v[k];
-    I.v[k] = st ? 0.0 : v;
-    I.x[k] += I.dt * v;
+    v[c] = I.sol[k];
+    v0[c] = I.v[k];
+    p[c] = I.vprev[k];
+    p2[c] = I.vprev2[k];
+    x[c] = I.x[k];
+  }
+#pragma unroll
+  for (int c = 0; c < 3; ++c) {
+    const int k = c * nv + row;
+    I.vprev3[k] = st ? 0.0 : p2[c];
+    I.vprev2[k] = st ? 0.0 : p[c];
+    I.vprev[k] = st ? 0.0 : v0[c];
+    I.v[k] = st ? 0.0 : v[c];
+    I.x[k] = x[c] + I.dt * v[c];
   }
   ROWS_END
 }
@@ -1591,7 +1656,8 @@ __device__ bool team_max_step(const Inst &I, Team &tm, double *out) {
   }
   if (!team_sync(tm)) return false;
   const double *part = I.part + 4 * (size_t)tm.bank * I.n_chunks;
-  tm.bank ^= 1;
+  __syncthreads();
+  if (threadIdx.x == 0) tm.bank ^= 1;
   if (threadIdx.x < 32) {
     double m = 0.0;
     for (int c = threadIdx.x; c < I.n_chunks; c += 32) m = fmax(m, __ldcg(part + 4 * c));
@@ -1894,39 +1960,39 @@ __device__ void load_descriptor(const Inst &src, Descriptor &d) {
 }
 
 // PREC: 0 = instances of either precision, 1 = FP64 instances only, 2 = FP32-refinement instances only.
-// MINB: CTAs per SM the register allocation is bounded for (the FP32 variant is compiled for 3, 4 and 5;
-// more resident warps mean more loads in flight, at the price of register spills; the autotuner picks).
+// MINB: CTAs per SM the register allocation is bounded for (the FP32 variant is compiled for 2, 3 and 4; more
+// resident warps mean more loads in flight, at the price of register spills; the autotuner picks between 3 and 4. With
+// every phase's loads issued ahead of its stores, 48 registers at 5 per SM lost to 64 at 4: batch of 256 34.4 against
+// 32.5 ms a call of 8 steps, 12 serving requests 14.3 against 13.1 ms (3 per SM: 36.0 and 12.0 ms)).
 // NT: the variant carries the Newton tangent (launched for batches with a Newton instance; the others run
 // variants without that code, whose register allocation it would otherwise burden).
 template <int PREC, int MINB, bool NT = false>
 __global__ void __launch_bounds__(kBlock, MINB) k_solve(const Inst *__restrict__ insts, Sched sch) {
-  Team tm;
-  tm.team = sch.cta_team[blockIdx.x];
-  if (tm.team < 0) return;
-  tm.rank = sch.cta_rank[blockIdx.x];
-  tm.size = sch.team_size[tm.team];
-  tm.bar = sch.bar + kBarWords * tm.team;
-  tm.abort_flag = sch.abort_flag;
-  tm.bank = 0;
-  tm.cluster = sch.cluster;
-  tm.cluster_ok = sch.cluster_ok;
-  tm.cap = sch.halo_cap;
-  tm.chord_k = sch.chord_k;
-  tm.wait_ns = sch.wait_ns;
-  if (tm.size == 1)
-    tm.mode = 0;
-  else if (sch.cluster > 0 && tm.size % sch.cluster == 0)
-    tm.mode = (tm.size == sch.cluster) ? 2 : 3;
-  else
-    tm.mode = 1;
+  // The team's state sits in shared memory (written by thread 0): in registers its fields would be live across every
+  // loop of the solver.
+  __shared__ Team tm;
+  const int team = sch.cta_team[blockIdx.x];
+  if (team < 0) return;
+  const int team_size = sch.team_size[team], team_rank = sch.cta_rank[blockIdx.x];
+  const int team_mode = team_size == 1 ? 0 : (sch.cluster > 0 && team_size % sch.cluster == 0) ? (team_size == sch.cluster ? 2 : 3) : 1;
+  if (threadIdx.x == 0) {
+    tm.team = team;
+    tm.bar = sch.bar + kBarWords * team;
+    tm.abort_flag = sch.abort_flag;
+    tm.bank = 0;
+    tm.cluster = sch.cluster;
+    tm.cluster_ok = sch.cluster_ok;
+    tm.cap = sch.halo_cap;
+    tm.chord_k = sch.chord_k;
+    tm.wait_ns = sch.wait_ns;
+  }
   // The team's own list first, then the shared queue of one-CTA instances, which every CTA serves once its
   // team's list is done (results do not depend on which CTA solves an instance). Both feed the same solver
   // call: a second, separately inlined call with the team size known to be 1 compiled to different rounding.
   __shared__ int s_q;
   __shared__ Descriptor s_desc;
-  const int q_end = sch.team_ptr[tm.team + 1];
-  int q = sch.team_ptr[tm.team];
-  const int team_size = tm.size, team_rank = tm.rank, team_mode = tm.mode;
+  const int q_end = sch.team_ptr[team + 1];
+  int q = sch.team_ptr[team];
   bool in_queue = false;
   for (;;) {
     int idx;
@@ -1934,7 +2000,7 @@ __global__ void __launch_bounds__(kBlock, MINB) k_solve(const Inst *__restrict__
       idx = sch.team_list[q++];
     } else {
       if (sch.n_queue <= 0) break;
-      if (threadIdx.x == 0) s_q = ld_volatile_i(tm.abort_flag) ? sch.n_queue : (int)atomicAdd(sch.queue_ctr, 1u);
+      if (threadIdx.x == 0) s_q = ld_volatile_i(sch.abort_flag) ? sch.n_queue : (int)atomicAdd(sch.queue_ctr, 1u);
       __syncthreads();
       const int qq = s_q;
       __syncthreads();
@@ -1942,15 +2008,18 @@ __global__ void __launch_bounds__(kBlock, MINB) k_solve(const Inst *__restrict__
       idx = sch.queue[qq];
       in_queue = true;
     }
-    tm.size = in_queue ? 1 : team_size;
-    tm.rank = in_queue ? 0 : team_rank;
-    tm.mode = in_queue ? 0 : team_mode;
     const InstStatus *stat = insts[idx].status;
     if (stat->err != SHELL_OK) continue;
     if (sch.chord_k > 0 && !(stat->nl_flags & 1)) continue;   // no chord iteration in progress
     load_descriptor(insts[idx], s_desc);
     const Inst &I = s_desc.inst;
-    tm.t0 = gtimer();
+    if (threadIdx.x == 0) {
+      tm.size = in_queue ? 1 : team_size;
+      tm.rank = in_queue ? 0 : team_rank;
+      tm.mode = in_queue ? 0 : team_mode;
+      tm.t0 = gtimer();
+    }
+    __syncthreads();
     bool ok;
     if (PREC == 1 || (PREC == 0 && I.precision == SHELL_FP64))
       ok = solve_fp64<NT>(I, tm);
@@ -1964,15 +2033,15 @@ __global__ void __launch_bounds__(kBlock, MINB) k_solve(const Inst *__restrict__
 
 }  // namespace
 
-// kernel of a precision mode and an occupancy variant (FP32: 3, 4 or 5 CTAs per SM; others: 2); prec 3: either
+// kernel of a precision mode and an occupancy variant (FP32: 2 to 4 CTAs per SM; others: 2); prec 3: either
 // precision with the Newton tangent
 typedef void (*SolveFn)(const Inst *, Sched);
 static SolveFn solve_fn(int prec, int occ) {
   if (prec == 3) return k_solve<0, 2, true>;
   if (prec == 2) {
-    if (occ >= 5) return k_solve<2, 5>;
-    if (occ == 4) return k_solve<2, 4>;
-    return k_solve<2, 3>;
+    if (occ >= 4) return k_solve<2, 4>;
+    if (occ == 3) return k_solve<2, 3>;
+    return k_solve<2, 2>;
   }
   if (prec == 1) return k_solve<1, 2>;
   return k_solve<0, 2>;
@@ -1982,14 +2051,13 @@ static SolveFn solve_fn(int prec, int occ) {
 // variant's CTAs per SM (228 KB per SM, 1 KB reserved per CTA). FP64-only launches stage nothing.
 int solve_halo_cap(int prec, int occ) {
   if (prec == 1) return 0;
-  if (prec == 2 && occ >= 5) return 2048;
-  if (prec == 2 && occ == 4) return 2880;
+  if (prec == 2 && occ >= 4) return 2880;
   return 4096;
 }
 
 static cudaError_t prepare_solve_fn(int prec, int occ) {
-  static bool done[4][6];
-  const int o = std::min(5, std::max(0, occ));
+  static bool done[4][5];
+  const int o = std::min(4, std::max(0, occ));
   if (done[prec][o]) return cudaSuccess;
   cudaError_t e = cudaFuncSetAttribute(solve_fn(prec, occ), cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        16 * solve_halo_cap(prec, occ));
@@ -2011,6 +2079,20 @@ int solve_blocks_per_sm(int prec, int occ) {
 // whole cluster (hardware co-schedules a cluster, and no team waits for CTAs outside its cluster); teams
 // larger than a cluster need the cooperative launch (all CTAs co-resident) and use global barriers.
 cudaError_t launch_solve(const Inst *d_insts, const Sched &sched, int grid, int prec, int occ, cudaStream_t st) {
+  // A grid that two CTAs per SM can hold takes the variant of 128 registers, which spills least: a spilled value is
+  // reloaded from L2, since the fence of each team barrier invalidates L1. (255 registers at one per SM, with a phase's
+  // first constant data loaded ahead of the barrier, measured the same: 128 x 128 cylinder 4.84 against 4.82 ms.)
+  if (prec == 2 && occ > 2 && sched.cluster == 0) {
+    static std::atomic<int> sms{0};
+    int n = sms.load();
+    if (n == 0) {
+      int dev = 0;
+      cudaGetDevice(&dev);
+      cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev);
+      sms.store(n);
+    }
+    if (grid <= 2 * n) occ = 2;
+  }
   cudaError_t e = prepare_solve_fn(prec, occ);
   if (e != cudaSuccess) return e;
   Sched sc = sched;
