@@ -906,9 +906,10 @@ __device__ void phase_spmv(const Inst &I, const Team &tm) {
 // In FP32 the recurrence r -= alpha s takes alpha rounded to FP32 while x takes the FP64 alpha, so x and the
 // recursive residual drift apart by about 2^-24 of each step; the FP64 residual of the next refinement round
 // is formed from x itself, so the drift is measured there and corrected like any other inner error.
+// sum: also writes the chunks' partials of ||r||^2 of the new r (the sums phase_spmv would form from it, see cg_loop).
 template <typename R>
 __device__ void phase_update(const Inst &I, const Team &tm, R alpha, R beta, bool first, double *x,
-                             double alpha_x) {
+                             double alpha_x, bool sum) {
   const int nv = I.nv;
   const bool amg = I.amg_levels > 0;
   const R *dinv = Vec<R>::dinv(I);
@@ -922,50 +923,59 @@ __device__ void phase_update(const Inst &I, const Team &tm, R alpha, R beta, boo
   typename Vec<R>::G *b0 = amg ? reinterpret_cast<typename Vec<R>::G *>(I.amg[0].b) : nullptr;
   typename Vec<R>::G *x0 = amg ? reinterpret_cast<typename Vec<R>::G *>(I.amg[0].x) : nullptr;
   const R om0 = amg ? LevelVal<R>::omega(I.amg[0]) : R(0);
-  ROWS_BEGIN(I, tm)
-  const R di = dinv[row];
-  // all loads before the first store: the stores may alias the next component's loads for all the compiler knows
-  R uo[3], ro[3], po[3], so[3], wo[3];
-  double xo[3];
-  if (amg) {
-    const typename Vec<R>::G gu = ldg4(g + row);
-    uo[0] = R(gu.x);
-    uo[1] = R(gu.y);
-    uo[2] = R(gu.z);
-  }
+  ChunkStage cs;
+  for (int ch = tm.rank; ch < I.n_chunks; ch += tm.size) {
+    R rr2 = R(0);
+    for (int rr = 0; rr < I.rows_per_thread; ++rr) {
+      const int row = (ch * I.rows_per_thread + rr) * kBlock + (int)threadIdx.x;
+      if (row >= nv) break;
+      const R di = dinv[row];
+      // all loads before the first store: the stores may alias the next component's loads for all the compiler knows
+      R uo[3], ro[3], po[3], so[3], wo[3];
+      double xo[3];
+      if (amg) {
+        const typename Vec<R>::G gu = ldg4(g + row);
+        uo[0] = R(gu.x);
+        uo[1] = R(gu.y);
+        uo[2] = R(gu.z);
+      }
 #pragma unroll
-  for (int c = 0; c < 3; ++c) {
-    const int k = c * nv + row;
-    ro[c] = r[k];
-    wo[c] = w[k];
-    if (!first) {
-      po[c] = p[k];
-      so[c] = s[k];
+      for (int c = 0; c < 3; ++c) {
+        const int k = c * nv + row;
+        ro[c] = r[k];
+        wo[c] = w[k];
+        if (!first) {
+          po[c] = p[k];
+          so[c] = s[k];
+        }
+        xo[c] = x[k];
+      }
+      R rv[3];
+#pragma unroll
+      for (int c = 0; c < 3; ++c) {
+        const int k = c * nv + row;
+        const R u = amg ? uo[c] : di * ro[c];
+        const R pc = first ? u : u + beta * po[c];
+        const R sc = first ? wo[c] : wo[c] + beta * so[c];
+        p[k] = pc;
+        s[k] = sc;
+        x[k] = xo[c] + alpha_x * double(pc);
+        const R rn = ro[c] - alpha * sc;
+        r[k] = rn;
+        rv[c] = rn;
+      }
+      if (!amg) {
+        g[row] = Vec<R>::mk(di * rv[0], di * rv[1], di * rv[2]);
+      } else {
+        b0[row] = Vec<R>::mk(rv[0], rv[1], rv[2]);
+        const R d = om0 * di;
+        x0[row] = Vec<R>::mk(d * rv[0], d * rv[1], d * rv[2]);
+      }
+      rr2 += rv[0] * rv[0] + rv[1] * rv[1] + rv[2] * rv[2];
     }
-    xo[c] = x[k];
+    if (sum) stage_chunk<R>(cs, I, tm, ch, R(0), R(0), rr2);
   }
-  R rv[3];
-#pragma unroll
-  for (int c = 0; c < 3; ++c) {
-    const int k = c * nv + row;
-    const R u = amg ? uo[c] : di * ro[c];
-    const R pc = first ? u : u + beta * po[c];
-    const R sc = first ? wo[c] : wo[c] + beta * so[c];
-    p[k] = pc;
-    s[k] = sc;
-    x[k] = xo[c] + alpha_x * double(pc);
-    const R rn = ro[c] - alpha * sc;
-    r[k] = rn;
-    rv[c] = rn;
-  }
-  if (!amg) {
-    g[row] = Vec<R>::mk(di * rv[0], di * rv[1], di * rv[2]);
-  } else {
-    b0[row] = Vec<R>::mk(rv[0], rv[1], rv[2]);
-    const R d = om0 * di;
-    x0[row] = Vec<R>::mk(d * rv[0], d * rv[1], d * rv[2]);
-  }
-  ROWS_END
+  if (cs.n) stage_flush(cs, I, tm);
 }
 
 // ------------------------------------------------------------------ multigrid V-cycle (preconditioner)
@@ -1523,7 +1533,9 @@ __device__ bool vcycle(const Inst &I, const Team &tm) {
 struct CgScalars {
   double alpha, beta, gamma, rho;
   float alpha32, beta32;
+  double rate;   // ||r||^2 reduction of the latest iteration (kept across the refinement rounds of a step)
   int verdict;   // 1: go on, 0: converged, -1: iteration cap, -3: not finite
+  int look;      // the coming update may meet the tolerance: its residual is summed at once
 };
 __device__ inline CgScalars &cg_state() {
   __shared__ CgScalars s;
@@ -1541,11 +1553,18 @@ struct CgCoef<double> {
   __device__ static double alpha(const CgScalars &s) { return s.alpha; }
   __device__ static double beta(const CgScalars &s) { return s.beta; }
 };
+// An iteration's end is seen in the residual its update leaves, but the sums of the next iteration, which tell, come
+// after another V-cycle and product. When the last reduction suggests that the coming update can meet the tolerance, its
+// residual is summed right away (one more reduction) and a converged solve ends there: the same test on the same sums.
+// The margin is wide (a factor 5 of the norm): a look in vain costs a reduction, a missed one a V-cycle and a product.
+constexpr double kLookAhead = 25.0;
 template <typename R>
 __device__ inline void cg_scalars(const double *sum, int it, double tol2, int max_it) {
   CgScalars &s = cg_state();
   const double gn = sum[0], dn = sum[1], rho = sum[2];
+  if (it > 0) s.rate = rho / s.rho;
   s.rho = rho;
+  s.look = rho * s.rate <= kLookAhead * tol2;
   if (!isfinite(rho) || !isfinite(gn) || !isfinite(dn)) {
     s.verdict = -3;
   } else if (rho <= tol2) {
@@ -1578,8 +1597,17 @@ __device__ int cg_loop(const Inst &I, Team &tm, double *x, double tol2, int max_
     const CgScalars &S = cg_state();
     *rho_out = S.rho;
     if (S.verdict <= 0) return S.verdict == 0 ? it : S.verdict;
-    phase_update<R>(I, tm, CgCoef<R>::alpha(S), CgCoef<R>::beta(S), it == 0, x, S.alpha);
+    const bool look = S.look && I.amg_levels > 0;
+    phase_update<R>(I, tm, CgCoef<R>::alpha(S), CgCoef<R>::beta(S), it == 0, x, S.alpha, look);
     if (!team_sync(tm)) return -2;
+    if (look) {
+      team_reduce(I, tm, red);
+      if (red[2] <= tol2) {
+        if (threadIdx.x == 0) cg_state().rate = red[2] / S.rho;
+        *rho_out = red[2];
+        return it + 1;
+      }
+    }
   }
 }
 
@@ -1839,6 +1867,7 @@ __device__ bool solve_fp64(const Inst &I, Team &tm) {
     if (!early) {
       // iteration k > 0: no need to solve below a tenth of the nonlinear target (inexact Newton)
       const double tol2 = fmax(I.pcg_rtol * I.pcg_rtol * ref, k > 0 ? nl_floor2(I) : 0.0);
+      if (threadIdx.x == 0) cg_state().rate = 1.0;
       iters = cg_loop<double, NT>(I, tm, I.sol, tol2, I.pcg_max_it, &rho);
       if (iters == -2) return false;
       if (iters < 0) {
@@ -1877,6 +1906,7 @@ __device__ bool solve_fp32r(const Inst &I, Team &tm) {
     return true;
   }
   int total = 0, rounds = 0;
+  if (threadIdx.x == 0) cg_state().rate = 1.0;
   double rel = 0.0, ref = bb;
   const bool writer = tm.rank == 0 && threadIdx.x == 0;   // the thread that reports rel (see cg_scalars on the others)
   bool early = false;
