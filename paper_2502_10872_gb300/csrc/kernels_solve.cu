@@ -138,19 +138,32 @@ __device__ bool team_sync(const Team &tm) {
   return s_ok != 0;
 }
 
-__device__ inline double warp_sum(double v) {
+// Sums of three values over the warp in one transposing butterfly: at the first two steps the lanes split the values
+// between them, so a lane does 6 additions and 6 shuffles instead of 15 each. Lane 8 k returns the sum of value k.
+// FP64 additions are what a reduction costs (2 lanes per clock and SM on GB300: 16 clocks per warp instruction).
+template <typename A>
+__device__ __forceinline__ A warp_sum3(A v0, A v1, A v2) {
+  const int lane = threadIdx.x & 31;
+  const bool hi = lane & 16, up = lane & 8;
+  A x = hi ? v2 : v0;
+  x += __shfl_xor_sync(0xffffffffu, hi ? v0 : v2, 16);
+  v1 += __shfl_xor_sync(0xffffffffu, v1, 16);
+  A y = !hi && up ? v1 : x;
+  y += __shfl_xor_sync(0xffffffffu, hi || up ? x : v1, 8);
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
-  return v;
+  for (int o = 4; o > 0; o >>= 1) y += __shfl_xor_sync(0xffffffffu, y, o);
+  return y;
 }
-__device__ inline float warp_sum(float v) {
+
+// Sums over the CTA's eight warps: lane 8 k + w holds warp w's sum of value k; lane 8 k returns the sum.
+__device__ __forceinline__ double octet_sum(double v) {
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
+  for (int o = kBlock / 64; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
   return v;
 }
 
-// Per-chunk partials: each chunk's three values are reduced by a fixed tree (warp shuffles, then the warps
-// in order). The warp sums of up to kStage chunks are staged in shared memory and written out together, so
+// Per-chunk partials: each chunk's three values are reduced by a fixed tree (warp shuffles, then the warps'
+// sums). The warp sums of up to kStage chunks are staged in shared memory and written out together, so
 // a CTA that owns several chunks of a phase pays two __syncthreads per kStage chunks instead of per chunk.
 constexpr int kStage = 32;
 
@@ -164,21 +177,17 @@ __device__ inline double (*stage_buf())[kBlock / 32][3] {
   return sm;
 }
 
+// A: the type the warp sums were staged in (FP32 sums are widened here: 24 lanes of one warp instead of one lane of
+// each warp and value)
+template <typename A>
 __device__ void stage_flush(ChunkStage &cs, const Inst &I, const Team &tm) {
-  double(*sm)[kBlock / 32][3] = stage_buf();
+  const A(*sm)[kBlock / 32][3] = reinterpret_cast<const A(*)[kBlock / 32][3]>(stage_buf());
+  const int lane = threadIdx.x & 31;
   __syncthreads();
-  if ((int)threadIdx.x < cs.n) {
-    const int k = threadIdx.x;
-    double a0 = sm[k][0][0], a1 = sm[k][0][1], a2 = sm[k][0][2];
-    for (int w = 1; w < kBlock / 32; ++w) {
-      a0 += sm[k][w][0];
-      a1 += sm[k][w][1];
-      a2 += sm[k][w][2];
-    }
-    double *dst = part_of(I, tm, cs.first + k * tm.size);
-    dst[0] = a0;
-    dst[1] = a1;
-    dst[2] = a2;
+  for (int k = threadIdx.x >> 5; k < cs.n; k += kBlock / 32) {   // a warp per chunk
+    double v = lane < 24 ? double(sm[k][lane & 7][lane >> 3]) : 0.0;
+    v = octet_sum(v);
+    if ((lane & 7) == 0 && lane < 24) part_of(I, tm, cs.first + k * tm.size)[lane >> 3] = v;
   }
   __syncthreads();
   cs.n = 0;
@@ -186,18 +195,12 @@ __device__ void stage_flush(ChunkStage &cs, const Inst &I, const Team &tm) {
 
 template <typename A>
 __device__ void stage_chunk(ChunkStage &cs, const Inst &I, const Team &tm, int ch, A v0, A v1, A v2) {
-  double(*sm)[kBlock / 32][3] = stage_buf();
+  A(*sm)[kBlock / 32][3] = reinterpret_cast<A(*)[kBlock / 32][3]>(stage_buf());
   if (cs.n == 0) cs.first = ch;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  v0 = warp_sum(v0);
-  v1 = warp_sum(v1);
-  v2 = warp_sum(v2);
-  if (lane == 0) {
-    sm[cs.n][warp][0] = double(v0);
-    sm[cs.n][warp][1] = double(v1);
-    sm[cs.n][warp][2] = double(v2);
-  }
-  if (++cs.n == kStage) stage_flush(cs, I, tm);
+  const A v = warp_sum3(v0, v1, v2);
+  if ((lane & 7) == 0 && lane < 24) sm[cs.n][warp][lane >> 3] = v;
+  if (++cs.n == kStage) stage_flush<A>(cs, I, tm);
 }
 
 // sum all chunk partials of an instance in a fixed order; result broadcast to the CTA. Flips the bank, so
@@ -212,45 +215,36 @@ __device__ __forceinline__ void team_reduce(const Inst &I, Team &tm, double out[
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   // every thread takes the chunks c, c + 256, ...; the threads of a warp are added by a tree, then the warps (one warp
   // alone takes up to 32 chunks). One warp summing all 1,024 chunks of the 512 x 512 plate spent 16 us per reduction on 32
-  // dependent rounds of L2 loads.
+  // dependent rounds of L2 loads. Warps without a chunk add nothing: their FP64 additions would occupy the pipe.
   const bool wide = n_chunks > 32;
-  double a0 = 0.0, a1 = 0.0, a2 = 0.0;
-  if (wide || warp == 0) {
-    for (int c = threadIdx.x; c < n_chunks; c += kBlock) {
+  double v = 0.0;
+  if (warp * 32 < n_chunks) {
+    double a0 = 0.0, a1 = 0.0, a2 = 0.0;
+    if ((int)threadIdx.x < n_chunks) {
+      const double *q = part + 4 * threadIdx.x;
+      a0 = __ldcg(q);
+      a1 = __ldcg(q + 1);
+      a2 = __ldcg(q + 2);
+    }
+    for (int c = threadIdx.x + kBlock; c < n_chunks; c += kBlock) {
       a0 += __ldcg(part + 4 * c);
       a1 += __ldcg(part + 4 * c + 1);
       a2 += __ldcg(part + 4 * c + 2);
     }
-    a0 = warp_sum(a0);
-    a1 = warp_sum(a1);
-    a2 = warp_sum(a2);
+    v = warp_sum3(a0, a1, a2);
   }
   if (wide) {
-    if (lane == 0) {
-      wsum[warp][0] = a0;
-      wsum[warp][1] = a1;
-      wsum[warp][2] = a2;
-    }
+    if ((lane & 7) == 0 && lane < 24) wsum[warp][lane >> 3] = v;
     __syncthreads();
-    if (warp == 0) {
-      const bool in = lane < kBlock / 32;
-      a0 = in ? wsum[lane][0] : 0.0;
-      a1 = in ? wsum[lane][1] : 0.0;
-      a2 = in ? wsum[lane][2] : 0.0;
-#pragma unroll
-      for (int o = kBlock / 64; o > 0; o >>= 1) {
-        a0 += __shfl_down_sync(0xffffffffu, a0, o);
-        a1 += __shfl_down_sync(0xffffffffu, a1, o);
-        a2 += __shfl_down_sync(0xffffffffu, a2, o);
-      }
-    }
+    if (warp == 0) v = octet_sum(lane < 24 ? wsum[lane & 7][lane >> 3] : 0.0);
   }
-  if (threadIdx.x == 0) {
-    res[0] = a0;
-    res[1] = a1;
-    res[2] = a2;
-    tm.bank ^= 1;   // the partials' readers of this CTA have read theirs
-    then(res);
+  if (warp == 0) {
+    if ((lane & 7) == 0 && lane < 24) res[lane >> 3] = v;
+    __syncwarp();
+    if (lane == 0) {
+      tm.bank ^= 1;   // the partials' readers of this CTA have read theirs
+      then(res);
+    }
   }
   __syncthreads();
   out[0] = res[0];
@@ -668,7 +662,7 @@ __device__ void phase_history(const Inst &I, const Team &tm) {
     }
     stage_chunk<double>(cs, I, tm, ch, e0, e1, e2);
   }
-  if (cs.n) stage_flush(cs, I, tm);
+  if (cs.n) stage_flush<double>(cs, I, tm);
 }
 
 // b = M v + dt (f + f_ext) (zero at pinned vertices and fixed components); warm start sol = the velocity extrapolated
@@ -755,7 +749,7 @@ __device__ void phase_rhs(const Inst &I, const Team &tm, int order) {
     }
     stage_chunk<double>(cs, I, tm, ch, bb, 0.0, 0.0);
   }
-  if (cs.n) stage_flush(cs, I, tm);
+  if (cs.n) stage_flush<double>(cs, I, tm);
 }
 
 // FP64 residual r64 = b - A64 sol; returns partial ||r64||^2. If R is float also prepares the inner CG:
@@ -830,7 +824,7 @@ __device__ void phase_resid(const Inst &I, const Team &tm) {
     }
     stage_chunk<double>(cs, I, tm, ch, rr2, 0.0, 0.0);
   }
-  if (cs.n) stage_flush(cs, I, tm);
+  if (cs.n) stage_flush<double>(cs, I, tm);
 }
 
 // w = A u (u = g); partials (r,u), (w,u), (r,r)
@@ -896,7 +890,7 @@ __device__ void phase_spmv(const Inst &I, const Team &tm) {
     }
     stage_chunk<R>(cs, I, tm, ch, gu, wu, rr2);
   }
-  if (cs.n) stage_flush(cs, I, tm);
+  if (cs.n) stage_flush<R>(cs, I, tm);
 }
 
 // p = u + beta p; s = w + beta s; x += alpha p; r -= alpha s; then (Jacobi) u = D^-1 r -> g. With the
@@ -971,11 +965,11 @@ __device__ void phase_update(const Inst &I, const Team &tm, R alpha, R beta, boo
         const R d = om0 * di;
         x0[row] = Vec<R>::mk(d * rv[0], d * rv[1], d * rv[2]);
       }
-      rr2 += rv[0] * rv[0] + rv[1] * rv[1] + rv[2] * rv[2];
+      if (sum) rr2 += rv[0] * rv[0] + rv[1] * rv[1] + rv[2] * rv[2];
     }
     if (sum) stage_chunk<R>(cs, I, tm, ch, R(0), R(0), rr2);
   }
-  if (cs.n) stage_flush(cs, I, tm);
+  if (cs.n) stage_flush<R>(cs, I, tm);
 }
 
 // ------------------------------------------------------------------ multigrid V-cycle (preconditioner)
@@ -1448,7 +1442,8 @@ __device__ bool dense_level(const Inst &I, const Team &tm) {
   const int n = I.amg_dense_n;
   const int per = (n + tm.size - 1) / tm.size;
   const int r0 = tm.rank * per, r1 = min(n, r0 + per);
-  double(*part)[kBlock / 32][3] = stage_buf();   // [32 rows][8 warps][3], free between reductions
+  // [32 rows][8 warps][3] in the solve precision, free between reductions
+  R(*part)[kBlock / 32][3] = reinterpret_cast<R(*)[kBlock / 32][3]>(stage_buf());
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   // b staged in shared memory (FP32) while the first columns are on their way; the next U columns are loaded before
   // the present ones are used
@@ -1490,16 +1485,17 @@ __device__ bool dense_level(const Inst &I, const Team &tm) {
 #pragma unroll
       for (int u = 0; u < U; ++u) a[u] = an[u];
     }
-    part[lane][w][0] = double(ax);
-    part[lane][w][1] = double(ay);
-    part[lane][w][2] = double(az);
+    part[lane][w][0] = ax;
+    part[lane][w][1] = ay;
+    part[lane][w][2] = az;
     __syncthreads();
     if (w == 0 && i < r1) {
-      R sx = R(part[lane][0][0]), sy = R(part[lane][0][1]), sz = R(part[lane][0][2]);
+      R sx = part[lane][0][0], sy = part[lane][0][1], sz = part[lane][0][2];
+#pragma unroll
       for (int g = 1; g < kBlock / 32; ++g) {
-        sx += R(part[lane][g][0]);
-        sy += R(part[lane][g][1]);
-        sz += R(part[lane][g][2]);
+        sx += part[lane][g][0];
+        sy += part[lane][g][1];
+        sz += part[lane][g][2];
       }
       y[i] = Vec<R>::mk(sx, sy, sz);
     }
