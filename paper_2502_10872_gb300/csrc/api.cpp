@@ -525,6 +525,35 @@ int launch_step(shell_batch *b) {
   return SHELL_OK;
 }
 
+// A step that may take many Newton or chord iterations (a quasi-static solve allows 1,000) is launched in groups, and
+// ends after the group in which its last instance stopped: the cantilever's 48 iterations took 1,001 pairs of
+// launches, recorded into a graph again on every call. A group costs one read of the statuses, about as much as two
+// launches of instances that are done, so it pays from a few times that many on.
+constexpr int kChordGroup = 12;
+int launch_step_groups(shell_batch *b) {
+  cudaStream_t st = b->mem.st;
+  std::vector<InstStatus> now(b->n_active);
+  for (int k = 0; k < b->chord_max;) {
+    const int end = std::min(k + kChordGroup, b->chord_max);
+    for (; k < end; ++k) {
+      CK(launch_forces(b->d_insts, b->d_tiles64, b->n_tiles64, 0, 0, st, k));
+      CK(solve_launch(b, st, k));
+    }
+    if (k == b->chord_max) break;
+    bool more = false;
+    for (int q = 0; q < b->n_active; ++q) {
+      const Inst &I = b->slots[b->active[q]]->h;
+      now[q].err = SHELL_OK;
+      now[q].nl_flags = 0;
+      if (I.nl_max > k) CK(cudaMemcpyAsync(&now[q], I.status, sizeof(InstStatus), cudaMemcpyDeviceToHost, st));
+    }
+    CK(cudaStreamSynchronize(st));
+    for (const InstStatus &s : now) more = more || (s.err == SHELL_OK && (s.nl_flags & 1));
+    if (!more) break;
+  }
+  return SHELL_OK;
+}
+
 // capture one step into a CUDA graph (falls back to direct launches if capture is refused)
 void try_capture(shell_batch *b) {
   b->graph_tried = true;
@@ -624,7 +653,8 @@ int batch_step(shell_batch *b, int n_steps, shell_step_stats *stats, const doubl
   // statuses before the call (cumulative counters)
   std::vector<InstStatus> before(n), after(n);
   for (int k = 0; k < n; ++k) before[k] = b->slots[b->active[k]]->last_status;
-  if (!b->graph_tried) try_capture(b);
+  const bool groups = b->chord_max > 4 * kChordGroup;
+  if (!b->graph_tried && !groups) try_capture(b);
   if (xin) {   // after the capture, which records only the step
     int rc = enqueue_states(b, nullptr, nullptr, xin, vin);
     if (rc != SHELL_OK) return rc;
@@ -656,6 +686,9 @@ int batch_step(shell_batch *b, int n_steps, shell_step_stats *stats, const doubl
         CK(solve_launch(b, st, k));
         CK(cudaEventRecord(b->pev[e0 + 2], st));
       }
+    } else if (groups) {
+      int rc = launch_step_groups(b);
+      if (rc != SHELL_OK) return rc;
     } else if (b->gexec) {
       CK(cudaGraphLaunch(b->gexec, st));
     } else {
@@ -1156,6 +1189,19 @@ int shell_create(const shell_mesh *mesh, const shell_material *mat, int32_t mode
   for (int s0 = 0; s0 < nt; s0 += kForceBlock) h->tiles.push_back({0, 0, s0, std::min(kForceBlock, nt - s0)});
   for (int s0 = 0; s0 < ne; s0 += kForceBlock) h->tiles.push_back({0, 1, s0, std::min(kForceBlock, ne - s0)});
 
+  // the direct solve of Newton iterations, where its band fits shared memory (it also needs the factor's reciprocal
+  // pivots and one vector there); the rule and its reason stand with the kernel (direct_factor)
+  std::vector<int32_t> perm;
+  if (I.precision == SHELL_FP64 && nv <= kBlock) {
+    std::vector<uint8_t> skip(nv);
+    for (int i = 0; i < nv; ++i) skip[i] = fixb[i] == 7;
+    const int w = (3 * band_order(T, skip.data(), &perm) + 2) | 1;   // odd: column reads without bank conflicts
+    if ((size_t)3 * nv * (w + 3) <= (size_t)kDirectWords)
+      I.dir_w = w;
+    else
+      perm.clear();
+  }
+
   // ---- persistent block
   auto layout = [&](Carver &C) {
     I.x = C.take<double>(3 * (size_t)nv);
@@ -1221,6 +1267,7 @@ int shell_create(const shell_mesh *mesh, const shell_material *mat, int32_t mode
     I.g = C.take<double>(4 * (size_t)nv);
     I.part = C.take<double>(8 * (size_t)I.n_chunks);
     I.ebuf = C.take<double>(2 * (size_t)(nt + ne));
+    I.dir_perm = perm.empty() ? nullptr : C.take<int32_t>(nv);
     I.status = C.take<InstStatus>(1);
     I.err_flags = C.take<int32_t>(1);
     h->d_inst = C.take<Inst>(1);
@@ -1296,6 +1343,7 @@ int shell_create(const shell_mesh *mesh, const shell_material *mat, int32_t mode
   CKF(up(I.vprev3, v0.data(), 8 * v0.size()));
   CKF(up(I.pinned, pin.data(), nv));
   if (partial) CKF(up(I.fix, fixb.data(), nv));
+  CKF(up(I.dir_perm, perm.data(), 4 * perm.size()));
   CKF(up(I.t_idx, T.t_idx.data(), 4 * T.t_idx.size()));
   CKF(up(I.t_bc, T.t_bc.data(), T.t_bc.size()));
   CKF(up(I.e_idx, T.e_idx.data(), 4 * T.e_idx.size()));

@@ -315,4 +315,63 @@ int build_topology(int nv, int nt, const int32_t *tris, int n_clamped, const int
   return SHELL_OK;
 }
 
+int band_order(const HostTopo &T, const uint8_t *skip, std::vector<int32_t> *perm) {
+  const int nv = T.nv;
+  auto entry = [&](int i, int k) { return T.sl_col[T.sl_ptr[i / 32] + 32 * k + i % 32]; };
+  std::vector<std::vector<int32_t>> nb(nv);
+  for (int i = 0; i < nv; ++i) {
+    if (skip[i]) continue;
+    for (int k = 0; k < T.row_ptr[i + 1] - T.row_ptr[i]; ++k) {
+      const int j = entry(i, k);
+      if (j != i && !skip[j]) nb[i].push_back(j);
+    }
+  }
+  auto fewer = [&](int a, int b) { return nb[a].size() != nb[b].size() ? nb[a].size() < nb[b].size() : a < b; };
+  std::vector<int32_t> order, level(nv, -1);
+  std::vector<char> done(nv, 0);
+  // breadth-first from `root` over the vertices that are not done, neighbours by increasing degree; returns the order
+  auto sweep = [&](int root) {
+    std::vector<int32_t> q{root};
+    level[root] = 0;
+    for (size_t h = 0; h < q.size(); ++h) {
+      std::vector<int32_t> next;
+      for (int j : nb[q[h]])
+        if (!done[j] && level[j] < 0) {
+          level[j] = level[q[h]] + 1;
+          next.push_back(j);
+        }
+      std::sort(next.begin(), next.end(), fewer);
+      q.insert(q.end(), next.begin(), next.end());
+    }
+    return q;
+  };
+  for (int i = 0; i < nv; ++i) {
+    if (done[i]) continue;
+    int root = i, depth = -1;
+    std::vector<int32_t> q;
+    for (int pass = 0; pass < 8; ++pass) {   // towards a peripheral vertex: the far end of the last sweep
+      q = sweep(root);
+      const int far = level[q.back()];
+      if (far > depth && pass < 7) {
+        depth = far;
+        int best = q.back();
+        for (int j : q)
+          if (level[j] == far && fewer(j, best)) best = j;
+        root = best;
+        for (int j : q) level[j] = -1;
+        continue;
+      }
+      break;
+    }
+    for (int j : q) done[j] = 1;
+    order.insert(order.end(), q.begin(), q.end());
+  }
+  perm->assign(nv, 0);
+  for (int k = 0; k < nv; ++k) (*perm)[order[k]] = nv - 1 - k;
+  int band = 0;
+  for (int i = 0; i < nv; ++i)
+    for (int j : nb[i]) band = std::max(band, std::abs((*perm)[i] - (*perm)[j]));
+  return band;
+}
+
 }  // namespace shl

@@ -27,4 +27,8 @@ struct HostTopo {
 int build_topology(int nv, int nt, const int32_t *tris, int n_clamped, const int32_t *clamped, int model,
                    HostTopo *out);
 
+// Bandwidth-reducing order of the mesh's vertices (reverse Cuthill-McKee over the matrix structure; vertices with
+// skip[i] != 0 are not coupled to the others). perm[i]: position of vertex i. Returns the bandwidth in vertices.
+int band_order(const HostTopo &T, const uint8_t *skip, std::vector<int32_t> *perm);
+
 }  // namespace shl

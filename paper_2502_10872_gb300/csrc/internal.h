@@ -19,6 +19,7 @@ namespace shl {
 constexpr int kSlice = 32;          // SELL slice height (one warp)
 constexpr int kBlock = 256;         // threads of every CTA of the persistent solve kernel
 constexpr int kMaxAmgLevels = 12;   // multigrid levels of one instance (build_amg's limit)
+constexpr int kDirectWords = 8192;  // doubles of shared memory the direct Newton solve may use (the Newton variant's staging buffer)
 constexpr int kForceBlock = 128;    // threads of a force tile
 constexpr int kMaxTeamWaitMs = 4000;  // default bound of a team-barrier wait (Sched::wait_ns)
 constexpr int kBarWords = 64;       // barrier words per team (256 bytes): a 64-bit arrival counter at [0, 2),
@@ -163,6 +164,11 @@ struct Inst {
   void *g;                       // [nv][4] gathered vector in the solve precision
   double *part;                  // [n_chunks][4] reduction partials
   double *ebuf;                  // [nt + ne][2] per-stencil energies (bending, membrane)
+
+  // Newton iterations of small FP64 instances (dir_perm not null): the Newton matrix is factored as a band matrix
+  // of width dir_w (unknowns) in shared memory, vertex i at position dir_perm[i]
+  int32_t *dir_perm;             // [nv] bandwidth-reducing vertex order
+  int32_t dir_w, pad3;
 
   InstStatus *status;            // one per instance
   int32_t *err_flags;            // precompute error flags (degenerate / singular)

@@ -903,9 +903,10 @@ __device__ void phase_spmv(const Inst &I, const Team &tm) {
 // sum: also writes the chunks' partials of ||r||^2 of the new r (the sums phase_spmv would form from it, see cg_loop).
 template <typename R>
 __device__ void phase_update(const Inst &I, const Team &tm, R alpha, R beta, bool first, double *x,
-                             double alpha_x, bool sum) {
+                             double alpha_x, bool sum, bool direct) {
   const int nv = I.nv;
-  const bool amg = I.amg_levels > 0;
+  const bool amg = I.amg_levels > 0 && !direct;
+  const bool given = amg || direct;   // u = B r is in g
   const R *dinv = Vec<R>::dinv(I);
   typename Vec<R>::G *g = Vec<R>::g(I);
   R *r = reinterpret_cast<R *>(I.r);
@@ -927,7 +928,7 @@ __device__ void phase_update(const Inst &I, const Team &tm, R alpha, R beta, boo
       // all loads before the first store: the stores may alias the next component's loads for all the compiler knows
       R uo[3], ro[3], po[3], so[3], wo[3];
       double xo[3];
-      if (amg) {
+      if (given) {
         const typename Vec<R>::G gu = ldg4(g + row);
         uo[0] = R(gu.x);
         uo[1] = R(gu.y);
@@ -948,7 +949,7 @@ __device__ void phase_update(const Inst &I, const Team &tm, R alpha, R beta, boo
 #pragma unroll
       for (int c = 0; c < 3; ++c) {
         const int k = c * nv + row;
-        const R u = amg ? uo[c] : di * ro[c];
+        const R u = given ? uo[c] : di * ro[c];
         const R pc = first ? u : u + beta * po[c];
         const R sc = first ? wo[c] : wo[c] + beta * so[c];
         p[k] = pc;
@@ -958,9 +959,9 @@ __device__ void phase_update(const Inst &I, const Team &tm, R alpha, R beta, boo
         r[k] = rn;
         rv[c] = rn;
       }
-      if (!amg) {
+      if (!given) {
         g[row] = Vec<R>::mk(di * rv[0], di * rv[1], di * rv[2]);
-      } else {
+      } else if (amg) {
         b0[row] = Vec<R>::mk(rv[0], rv[1], rv[2]);
         const R d = om0 * di;
         x0[row] = Vec<R>::mk(d * rv[0], d * rv[1], d * rv[2]);
@@ -1521,6 +1522,148 @@ __device__ bool vcycle(const Inst &I, const Team &tm) {
   return true;
 }
 
+// ------------------------------------------------------------------ direct solve of small Newton systems
+// The Newton matrix of a thin strip is far from what the preconditioners approximate (the constant matrix: its
+// isotropic membrane block is as stiff across the sheet as along it): the cantilever of 51 nodes took 24,415 Jacobi-
+// preconditioned iterations over 48 Newton steps, each bound by the FP64 pipe of one SM. An FP64 instance of one row
+// block whose band fits the launch's staging buffer is solved by a band LDL^T factorisation of its assembled Newton
+// matrix instead, applied as the preconditioner of the same iteration: that keeps the stop test, and the product with
+// the matrix itself decides (one or two iterations a solve). The cantilever's call, with its launches in groups: 930 ->
+// 19.6 ms. Larger instances keep PCG: their factor would not fit, and would be one CTA's work.
+// Layout in shared memory: band [3 nv][dir_w + 1], row i's entry (i, j) at i (dir_w + 1) + j - i + dir_w, holding
+// L_ij d_j below the diagonal; reciprocal pivots [3 nv]; the vector being solved [3 nv].
+__device__ inline bool direct_on(const Inst &I, const Team &tm) {
+  return I.nl_newton && I.dir_perm && 3 * I.nv * (I.dir_w + 3) <= 2 * tm.cap;
+}
+
+// Assembles and factors (all threads of one CTA). Row by row: the step matrix, then the tangent blocks of the row's
+// triangles (see tangent_corr), block (a, b) = dt^2 A t sum_kl g_a^k g_b^l dP_k / dU_l. Returns false if a pivot is
+// not positive and finite.
+__device__ __noinline__ bool direct_factor(const Inst &I) {
+  __shared__ int s_bad;
+  const int nv = I.nv, n = 3 * nv, W = I.dir_w, ld = W + 1;
+  double *B = reinterpret_cast<double *>(sh_halo);
+  double *rcp = B + n * ld;
+  __syncthreads();   // earlier readers of the buffer are done
+  for (int e = threadIdx.x; e < n * ld; e += kBlock) B[e] = 0.0;
+  if (threadIdx.x == 0) s_bad = 0;
+  __syncthreads();
+  const int v = threadIdx.x;
+  if (v < nv) {
+    const int nt = I.nt, kt = I.kt, pv = 3 * I.dir_perm[v];
+    const unsigned fv = I.fix ? (unsigned)I.fix[v] : 0u;
+    auto at = [&](int c, int pu, int d) -> double & { return B[(pv + c) * ld + (pu + d - pv - c + W)]; };
+    const int s = v >> 5;
+    for (int p = I.sl_ptr[s] + (v & 31); p < I.sl_ptr[s + 1]; p += 32) {
+      const double a = I.val64[p];
+      const int u = I.sl_col[p], pu = 3 * I.dir_perm[u];
+      if (a == 0.0 || pu > pv) continue;
+      const unsigned fx = u == v ? 0u : fv | (I.fix ? (unsigned)I.fix[u] : 0u);   // fixed components: diagonal only
+      for (int c = 0; c < 3; ++c)
+        if (!((fx >> c) & 1u)) at(c, pu, c) += a;
+    }
+    const double mu = I.mu, lam = I.lam, w2 = 2.0 * (mu + lam), dt2 = I.dt * I.dt;
+    const double *T = I.m_T;
+    if (!I.pinned[v]) {
+      for (int q = I.vtx_ptr[v]; q < I.vtx_ptr[v + 1]; ++q) {
+        const int sl = I.vtx_slot[q];
+        if (sl >= nt * kt) continue;            // an edge stencil's slot
+        const int t = sl / kt, j = sl - t * kt;
+        if (j >= 3) continue;                   // a bending neighbour's slot
+        const double gp = I.m_D64[t], gq = I.m_D64[nt + t], gr = I.m_D64[2 * nt + t], sc = dt2 * I.m_At64[t];
+        const double g0[3] = {-gp, gp, 0.0}, g1[3] = {-gq - gr, gq, gr};
+        const v3<double> R0 = {T[t], T[nt + t], T[2 * nt + t]}, R1 = {T[3 * nt + t], T[4 * nt + t], T[5 * nt + t]};
+        const double kap = T[6 * nt + t], Q00 = T[7 * nt + t], Q01 = T[8 * nt + t], Q11 = T[9 * nt + t];
+        const v3<double> nn = cross(R0, R1);
+        const double r0[3] = {R0.x, R0.y, R0.z}, r1[3] = {R1.x, R1.y, R1.z}, nr[3] = {nn.x, nn.y, nn.z};
+        const double ga0 = sc * (j == 0 ? g0[0] : j == 1 ? g0[1] : g0[2]), ga1 = sc * (j == 0 ? g1[0] : j == 1 ? g1[1] : g1[2]);
+        for (int b = 0; b < 3; ++b) {
+          const int u = I.t_idx[b * nt + t], pu = 3 * I.dir_perm[u];
+          if (pu > pv || I.pinned[u]) continue;
+          const double gb0 = b == 0 ? g0[0] : b == 1 ? g0[1] : g0[2], gb1 = b == 0 ? g1[0] : b == 1 ? g1[1] : g1[2];
+          const double s00 = ga0 * gb0, s01 = ga0 * gb1, s10 = ga1 * gb0, s11 = ga1 * gb1;
+          const double c00 = s00 * (2.0 * mu + lam) + s11 * (mu + kap), c11 = s00 * (mu + kap) + s11 * (2.0 * mu + lam);
+          const double c01 = s10 * (mu - kap) + s01 * lam, c10 = s10 * lam + s01 * (mu - kap);
+          const double cn = s00 * Q00 + s11 * Q11 + (s01 + s10) * Q01, ci = w2 * (s00 + s11);
+          const unsigned fu = I.fix ? (unsigned)I.fix[u] : 0u;
+#pragma unroll
+          for (int c = 0; c < 3; ++c) {
+            const double x0 = c00 * r0[c] + c10 * r1[c], x1 = c01 * r0[c] + c11 * r1[c], xn = cn * nr[c];
+#pragma unroll
+            for (int d = 0; d < 3; ++d) {
+              if ((u == v && d > c) || ((fv >> c) & 1u) || ((fu >> d) & 1u)) continue;
+              at(c, pu, d) += x0 * r0[d] + x1 * r1[d] + xn * nr[d] - (c == d ? ci : 0.0);
+            }
+          }
+        }
+      }
+    }
+  }
+  __syncthreads();
+  // right-looking, one column a step: a warp per row of the trailing triangle; the thread that updates the next pivot
+  // also inverts it, so a step takes one barrier
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  if (threadIdx.x == 0) {
+    const double d = B[W];
+    if (!(d > 0.0) || !isfinite(d)) s_bad = 1;
+    rcp[0] = 1.0 / d;
+  }
+  __syncthreads();
+  for (int k = 0; k < n; ++k) {
+    const double rk = rcp[k];
+    const int last = min(k + W, n - 1);
+    for (int i = k + 1 + warp; i <= last; i += kBlock / 32) {
+      const double ci = B[i * ld + k - i + W];
+      if (ci == 0.0 && i != k + 1) continue;
+      const double li = ci * rk;
+      for (int j = k + 1 + lane; j <= i; j += 32) {
+        const double x = B[i * ld + j - i + W] - li * B[j * ld + k - j + W];
+        B[i * ld + j - i + W] = x;
+        if (i == k + 1) {
+          if (!(x > 0.0) || !isfinite(x)) s_bad = 1;
+          rcp[i] = 1.0 / x;
+        }
+      }
+    }
+    __syncthreads();
+  }
+  return s_bad == 0;
+}
+
+// g = J^-1 r with the factor in shared memory (all threads of the CTA; one warp runs the substitutions)
+__device__ __noinline__ void direct_apply(const Inst &I) {
+  const int nv = I.nv, n = 3 * nv, W = I.dir_w, ld = W + 1;
+  const double *B = reinterpret_cast<const double *>(sh_halo), *rcp = B + n * ld;
+  double *y = reinterpret_cast<double *>(sh_halo) + n * (ld + 1);
+  const double *r = reinterpret_cast<const double *>(I.r);
+  D4 *g = reinterpret_cast<D4 *>(I.g);
+  const int v = threadIdx.x;
+  int p = 0;
+  if (v < nv) {
+    p = 3 * I.dir_perm[v];
+    for (int c = 0; c < 3; ++c) y[p + c] = r[c * nv + v];
+  }
+  __syncthreads();
+  if (threadIdx.x < 32) {
+    const int lane = threadIdx.x;
+    for (int k = 0; k < n; ++k) {
+      const double t = y[k] * rcp[k];
+      const int last = min(k + W, n - 1);
+      for (int i = k + 1 + lane; i <= last; i += 32) y[i] -= B[i * ld + k - i + W] * t;
+      __syncwarp();
+    }
+    for (int k = n - 1; k >= 0; --k) {
+      const double t = y[k] * rcp[k];
+      __syncwarp();
+      if (lane == 0) y[k] = t;
+      for (int j = max(0, k - W) + lane; j < k; j += 32) y[j] -= B[k * ld + j - k + W] * t;
+      __syncwarp();
+    }
+  }
+  __syncthreads();
+  if (v < nv) g[v] = {y[p], y[p + 1], y[p + 2], 0.0};
+}
+
 // Scalars of the recurrence, computed by one thread of the CTA from the reduced sums and read by the others from
 // shared memory: three dependent FP64 divisions in every thread occupied the FP64 pipe (2 operations per clock and
 // SM on GB300) for several thousand clocks of each iteration. Per call, with the smoother's weight read in FP32
@@ -1584,8 +1727,25 @@ __device__ inline void cg_scalars(const double *sum, int it, double tol2, int ma
 template <typename R, bool NT>
 __device__ int cg_loop(const Inst &I, Team &tm, double *x, double tol2, int max_it, double *rho_out) {
   if (!team_sync(tm)) return -2;
+  bool direct = false;
+  if constexpr (NT && sizeof(R) == 8) {
+    if (direct_on(I, tm)) {   // one row block: the team's first CTA factors and solves
+      if (tm.rank == 0) {
+        const bool ok = direct_factor(I);
+        if (threadIdx.x == 0) reinterpret_cast<double *>(I.w)[0] = ok ? 1.0 : 0.0;   // w is free until the first product
+      }
+      if (!team_sync(tm)) return -2;
+      direct = __ldcg(reinterpret_cast<const double *>(I.w)) != 0.0;
+    }
+  }
   for (int it = 0;; ++it) {
-    if (I.amg_levels > 0 && !vcycle<R, NT>(I, tm)) return -2;
+    if (direct) {
+      if constexpr (NT && sizeof(R) == 8)
+        if (tm.rank == 0) direct_apply(I);
+      if (!team_sync(tm)) return -2;
+    } else if (I.amg_levels > 0 && !vcycle<R, NT>(I, tm)) {
+      return -2;
+    }
     phase_spmv<R, NT>(I, tm);
     if (!team_sync(tm)) return -2;
     double red[3];
@@ -1593,8 +1753,8 @@ __device__ int cg_loop(const Inst &I, Team &tm, double *x, double tol2, int max_
     const CgScalars &S = cg_state();
     *rho_out = S.rho;
     if (S.verdict <= 0) return S.verdict == 0 ? it : S.verdict;
-    const bool look = S.look && I.amg_levels > 0;
-    phase_update<R>(I, tm, CgCoef<R>::alpha(S), CgCoef<R>::beta(S), it == 0, x, S.alpha, look);
+    const bool look = direct || (S.look && I.amg_levels > 0);
+    phase_update<R>(I, tm, CgCoef<R>::alpha(S), CgCoef<R>::beta(S), it == 0, x, S.alpha, look, direct);
     if (!team_sync(tm)) return -2;
     if (look) {
       team_reduce(I, tm, red);
