@@ -127,6 +127,7 @@ struct shell_handle {
   void *amg_block = nullptr;     // multigrid hierarchy (device), if any
   size_t amg_bytes = 0;
   int64_t vcycle_bytes = 0;      // algorithmic bytes of one FP32 V-cycle
+  int units = 0;                 // most units any phase of a step splits into (see rebuild_tables)
   double est_iters = 64.0;       // scheduling estimate (PCG iterations per step)
   long long meas_ns = 0;         // longest device solve time of the last call's steps (0 = never run)
   int meas_team = 0;             // team size it ran with
@@ -386,6 +387,18 @@ int rebuild_tables(shell_batch *b) {
         team_inst.push_back({k});
         used += team_size.back();
       }
+    }
+    // An instance alone leaves SMs idle: phases that split into more units than row blocks (forces, the down step's
+    // residual and restriction blocks, the dense level's rows) get a CTA per unit, as far as the CTAs per SM that its
+    // row blocks take anyway reach (more would only lengthen the barriers). With the dense level's split among many
+    // CTAs (dense_level), per call: 24 x 17 panel in FP64 958 -> 737 us, 97 x 62 Jacobi case 780 -> 678 us, 128 x 128
+    // cylinder 4.33 -> 3.94 ms, in FP64 7.38 -> 6.15 ms, 512 x 512 plate 13.1 -> 12.2 ms.
+    if (n == 1 && team_size.size() == 1) {
+      const int sms = num_sms(), blocks = cmax(0);
+      const int per_sm = std::min(occ, (blocks + sms - 1) / sms);
+      const int c = std::min(std::max(blocks, b->slots[b->active[0]]->units), sms * per_sm);
+      used += std::max(0, c - team_size[0]);
+      team_size[0] = std::max(team_size[0], c);
     }
     // the one-CTA instances are not bound to the bins the plan sized: they form a queue in decreasing work,
     // served by one-CTA workers (every CTA the multi-CTA teams leave, at least as many as the bins) and by the
@@ -911,6 +924,11 @@ int setup_amg(shell_handle *h, const HostTopo &T, int mode, bool stage, const st
   }
   h->vcycle_bytes += 136 * (int64_t)H.levels[top].A.n;
   h->vcycle_bytes += 4 * (int64_t)(H.dense_level > 0 ? H.dense.size() : H.coarse_inv.size());
+  for (int l = 0; l < top; ++l) {   // down step: residual blocks and restriction blocks of 64 rows (level 0: 256)
+    const int n = H.levels[l].A.n, nn = H.levels[l + 1].A.n, per = kBlock / 4;
+    h->units = std::max(h->units, (l == 0 ? (n + kBlock - 1) / kBlock : (n + per - 1) / per) + (nn + per - 1) / per);
+  }
+  if (H.dense_level > 0) h->units = std::max(h->units, (H.dense_n + 7) / 8);
   std::vector<HostSell> As(L), Ps(L), Rs(L);
   for (int l = 0; l < L; ++l) {
     if (l > 0) As[l] = to_sell4(H.levels[l].A);
@@ -1177,6 +1195,7 @@ int shell_create(const shell_mesh *mesh, const shell_material *mat, int32_t mode
   I.lam = mat->E * mat->nu / (1.0 - mat->nu * mat->nu);
   I.n_slots = T.n_slots;
   I.n_local = T.n_local;
+  if (I.precision != SHELL_FP64) h->units = (nt + T.ne + kBlock - 1) / kBlock;   // forces in the step kernel
   const size_t nnz_pad = (size_t)T.sl_ptr[T.n_slices];
   h->nnz = T.nnz;
   h->nnz_pad = (int64_t)nnz_pad;

@@ -1428,17 +1428,19 @@ __device__ bool up_step(const Inst &I, int l, const Team &tm) {
 
 // y_d = B b_d on the dense level d: B is the cycle of levels >= d (started from zero), a fixed linear map
 // set up on the host as a dense column-major matrix. This replaces that part of the cycle, a chain of
-// small dependent phases, by one product. Rows are split into contiguous chunks, one per CTA of the team;
-// inside a CTA, warp w sums the columns j = w, w + 8, ... in increasing order for 32 consecutive rows
-// (coalesced column reads of B), and the eight partial sums of a row are added in warp order: the same
-// operations whatever the team size.
+// small dependent phases, by one product. Rows are split into contiguous chunks, one per CTA of the team. A row's
+// sum has 32 parts, part p the columns j = p, p + 32, ... in increasing order; a warp adds four of them pairwise, and
+// the eight warps' sums are added in warp order: the same operations whatever the team size. A CTA of up to 8 rows (a
+// large team) gives each row four lanes of every warp, one part each; otherwise a lane takes a row and the four parts
+// in turn. (A lane per row throughout left 26 of 32 lanes idle where 66 CTAs share 351 rows: 7.2 k clocks, and in
+// FP64, where an instruction costs the pipe 16 clocks for any number of active lanes, 25 k.)
 template <typename R>
 __device__ bool dense_level(const Inst &I, const Team &tm) {
   typedef typename Vec<R>::G G;
   constexpr int U = 8;
   const AmgDev &D = I.amg[I.amg_dense_level];
   const G *b = reinterpret_cast<const G *>(D.b);
-  G *y = reinterpret_cast<G *>(D.y);
+  R *y = reinterpret_cast<R *>(D.y);
   const R *B = LevelVal<R>::dense(I);
   const int n = I.amg_dense_n;
   const int per = (n + tm.size - 1) / tm.size;
@@ -1446,17 +1448,23 @@ __device__ bool dense_level(const Inst &I, const Team &tm) {
   // [32 rows][8 warps][3] in the solve precision, free between reductions
   R(*part)[kBlock / 32][3] = reinterpret_cast<R(*)[kBlock / 32][3]>(stage_buf());
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const bool quad = per <= 8;
+  const int rows = quad ? 8 : 32;   // rows of a pass
+  const int i0 = quad ? lane >> 2 : lane;
+  // column of load k: one part's columns are 32 apart; a lane with a row of its own takes its warp's four parts in turn
+  auto col = [&](int k) { return quad ? 4 * w + (lane & 3) + 32 * k : 4 * w + (k & 3) + 32 * (k >> 2); };
+  const int nk = (quad ? 1 : 4) * ((n + 31) / 32);   // loads per lane
   // b staged in shared memory (FP32) while the first columns are on their way; the next U columns are loaded before
   // the present ones are used
   R a[U], an[U];
-  auto columns = [&](R *to, int i, int j0) {
+  auto columns = [&](R *to, int i, int k0) {
 #pragma unroll
     for (int u = 0; u < U; ++u) {
-      const int j = j0 + 8 * u;
-      to[u] = (i < r1 && j < n) ? B[(size_t)j * n + i] : R(0);
+      const int j = col(k0 + u);
+      to[u] = (i < r1 && k0 + u < nk && j < n) ? B[(size_t)j * n + i] : R(0);
     }
   };
-  columns(a, r0 + lane, w);
+  columns(a, r0 + i0, 0);
   bool st = false;
   if constexpr (sizeof(R) == 4) {
     st = n <= tm.cap;
@@ -1465,40 +1473,57 @@ __device__ bool dense_level(const Inst &I, const Team &tm) {
       __syncthreads();
     }
   }
-  for (int base = r0; base < r1; base += 32) {
-    const int i = base + lane;
-    if (base != r0) columns(a, i, w);
-    R ax = R(0), ay = R(0), az = R(0);
-    for (int j0 = w; j0 < n; j0 += 8 * U) {
-      if (j0 + 8 * U < n) columns(an, i, j0 + 8 * U);
+  for (int base = r0; base < r1; base += rows) {
+    const int i = base + i0;
+    if (base != r0) columns(a, i, 0);
+    R s[4][3] = {};   // parts (one of them with four lanes a row)
+    for (int k0 = 0; k0 < nk; k0 += U) {
+      if (k0 + U < nk) columns(an, i, k0 + U);
 #pragma unroll
       for (int u = 0; u < U; ++u) {
-        const int j = j0 + 8 * u < n ? j0 + 8 * u : 0;
+        const int jc = col(k0 + u), j = jc < n ? jc : 0;
         G t;
         if constexpr (sizeof(R) == 4)
           t = st ? sh_halo[j] : b[j];
         else
           t = ldg4(b + j);
-        ax += a[u] * R(t.x);
-        ay += a[u] * R(t.y);
-        az += a[u] * R(t.z);
+        const R av = a[u];
+        if (quad) {
+          s[0][0] += av * R(t.x);
+          s[0][1] += av * R(t.y);
+          s[0][2] += av * R(t.z);
+        } else {
+          s[u & 3][0] += av * R(t.x);
+          s[u & 3][1] += av * R(t.y);
+          s[u & 3][2] += av * R(t.z);
+        }
       }
 #pragma unroll
       for (int u = 0; u < U; ++u) a[u] = an[u];
     }
-    part[lane][w][0] = ax;
-    part[lane][w][1] = ay;
-    part[lane][w][2] = az;
-    __syncthreads();
-    if (w == 0 && i < r1) {
-      R sx = part[lane][0][0], sy = part[lane][0][1], sz = part[lane][0][2];
+    R v[3];
 #pragma unroll
-      for (int g = 1; g < kBlock / 32; ++g) {
-        sx += part[lane][g][0];
-        sy += part[lane][g][1];
-        sz += part[lane][g][2];
+    for (int c = 0; c < 3; ++c) {
+      if (quad) {
+        v[c] = s[0][c];
+        v[c] += __shfl_xor_sync(0xffffffffu, v[c], 1);
+        v[c] += __shfl_xor_sync(0xffffffffu, v[c], 2);
+      } else {
+        v[c] = (s[0][c] + s[1][c]) + (s[2][c] + s[3][c]);
       }
-      y[i] = Vec<R>::mk(sx, sy, sz);
+    }
+    if (!quad || (lane & 3) == 0) {
+      part[i0][w][0] = v[0];
+      part[i0][w][1] = v[1];
+      part[i0][w][2] = v[2];
+    }
+    __syncthreads();
+    const int io = base + lane;
+    if (w < 3 && lane < rows && io < r1) {   // a warp per component
+      R sum = part[lane][0][w];
+#pragma unroll
+      for (int g = 1; g < kBlock / 32; ++g) sum += part[lane][g][w];
+      y[4 * io + w] = sum;
     }
     __syncthreads();
   }
