@@ -424,6 +424,89 @@ void build_amg(const HostCsr &A0, HostAmg *out, int max_levels, int coarse_max, 
   }
 }
 
+bool band_inverse(const HostCsr &A, const std::vector<int32_t> &perm, int band, double eps, std::vector<double> *inv) {
+  const int n = A.n, w = band + 1;
+  std::vector<double> sd(n);   // sqrt of the diagonal, by position
+  std::vector<int32_t> at(n);  // row at a position
+  for (int i = 0; i < n; ++i) at[perm[i]] = i;
+  for (int i = 0; i < n; ++i) {
+    const double d = diag_of(A, i);
+    if (!(d > 0)) return false;
+    sd[perm[i]] = std::sqrt(d);
+  }
+  // L[i][j - i + band], j <= i: the scaled matrix, then its factor
+  std::vector<double> L((size_t)n * w, 0.0);
+  double snorm = 0.0;
+  for (int i = 0; i < n; ++i) {
+    const int pi = perm[i];
+    double rs = 0.0;
+    for (int q = A.ptr[i]; q < A.ptr[i + 1]; ++q) {
+      const int pj = perm[A.col[q]];
+      const double v = A.val[q] / (sd[pi] * sd[pj]);
+      rs += std::fabs(v);
+      if (pj > pi || A.val[q] == 0.0) continue;
+      if (pi - pj > band) return false;
+      L[(size_t)pi * w + pj - pi + band] = v;
+    }
+    snorm = std::max(snorm, rs);
+  }
+  std::vector<double> rd(n);
+  for (int i = 0; i < n; ++i) {
+    double *li = &L[(size_t)i * w] - i + band;
+    for (int j = std::max(0, i - band); j <= i; ++j) {
+      const double *lj = &L[(size_t)j * w] - j + band;
+      double t = li[j];
+      for (int k = std::max(0, i - band); k < j; ++k) t -= li[k] * lj[k];
+      if (j < i) {
+        li[j] = t * rd[j];
+      } else {
+        if (!(t > 0)) return false;
+        li[i] = std::sqrt(t);
+        rd[i] = 1.0 / li[i];
+      }
+    }
+  }
+  // K unit vectors at a time; the inverse is symmetric, so a column is needed from its own position down only
+  constexpr int K = 8;
+  std::vector<double> Y((size_t)n * K);
+  inv->assign((size_t)n * n, 0.0);
+  double cnorm = 0.0;
+  std::vector<double> rs(n, 0.0);
+  for (int c0 = 0; c0 < n; c0 += K) {
+    std::fill(Y.begin() + (size_t)c0 * K, Y.end(), 0.0);
+    for (int c = 0; c < K && c0 + c < n; ++c) Y[(size_t)(c0 + c) * K + c] = 1.0;
+    for (int i = c0; i < n; ++i) {
+      const double *li = &L[(size_t)i * w] - i + band;
+      double t[K];
+      for (int c = 0; c < K; ++c) t[c] = Y[(size_t)i * K + c];
+      for (int k = std::max(c0, i - band); k < i; ++k)
+        for (int c = 0; c < K; ++c) t[c] -= li[k] * Y[(size_t)k * K + c];
+      for (int c = 0; c < K; ++c) Y[(size_t)i * K + c] = t[c] * rd[i];
+    }
+    for (int i = n - 1; i >= c0; --i) {
+      double t[K];
+      for (int c = 0; c < K; ++c) t[c] = Y[(size_t)i * K + c];
+      for (int k = i + 1; k <= std::min(n - 1, i + band); ++k) {
+        const double l = L[(size_t)k * w + i - k + band];
+        for (int c = 0; c < K; ++c) t[c] -= l * Y[(size_t)k * K + c];
+      }
+      for (int c = 0; c < K; ++c) Y[(size_t)i * K + c] = t[c] * rd[i];
+    }
+    for (int c = 0; c < K && c0 + c < n; ++c) {
+      const int p = c0 + c;
+      for (int i = p; i < n; ++i) {
+        const double y = Y[(size_t)i * K + c], v = y / (sd[i] * sd[p]);
+        (*inv)[(size_t)at[p] * n + at[i]] = v;
+        (*inv)[(size_t)at[i] * n + at[p]] = v;
+        rs[i] += std::fabs(y);
+        if (i != p) rs[p] += std::fabs(y);
+      }
+    }
+  }
+  for (double v : rs) cnorm = std::max(cnorm, v);
+  return std::isfinite(cnorm) && eps * cnorm * snorm <= 0.25;
+}
+
 HostSell to_sell4(const HostCsr &M) {
   HostSell S;
   S.n = M.n;

@@ -49,6 +49,12 @@ struct HostAmg {
 void build_amg(const HostCsr &A, HostAmg *out, int max_levels = 12, int coarse_max = 48, double theta = 0.08,
                int dense_max = 400);
 
+// Inverse of the SPD matrix A (n x n, row-major = column-major) by a band Cholesky factorisation in the order perm
+// (row i at position perm[i]; band: largest distance of coupled rows). False if a pivot is not positive, or if the
+// inverse's entries rounded to a relative eps could leave it indefinite: eps ||C||_inf ||S||_inf > 1/4, S the matrix
+// with unit diagonal and C its inverse (entrywise rounding is invariant under that scaling).
+bool band_inverse(const HostCsr &A, const std::vector<int32_t> &perm, int band, double eps, std::vector<double> *inv);
+
 HostSell to_sell(const HostCsr &M);
 
 // SELL with 4 lanes per row (for the long rows of the restriction): slices of 8 rows; entry k of the slice's

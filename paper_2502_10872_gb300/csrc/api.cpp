@@ -229,6 +229,8 @@ void destroy_graph(shell_batch *b) {
   b->graph_tried = false;
 }
 
+constexpr int kDenseTeamRows = 128;   // rows from which a dense inverse is worth a team of CTAs (four passes of one CTA)
+
 // The step kernel's variant with the Newton tangent also carries the projection of per-component constraints.
 static bool uses_nt_variant(const Inst &I) { return (I.nl_newton && I.nl_max > 1) || I.fix != nullptr; }
 
@@ -388,18 +390,6 @@ int rebuild_tables(shell_batch *b) {
         used += team_size.back();
       }
     }
-    // An instance alone leaves SMs idle: phases that split into more units than row blocks (forces, the down step's
-    // residual and restriction blocks, the dense level's rows) get a CTA per unit, as far as the CTAs per SM that its
-    // row blocks take anyway reach (more would only lengthen the barriers). With the dense level's split among many
-    // CTAs (dense_level), per call: 24 x 17 panel in FP64 958 -> 737 us, 97 x 62 Jacobi case 780 -> 678 us, 128 x 128
-    // cylinder 4.33 -> 3.94 ms, in FP64 7.38 -> 6.15 ms, 512 x 512 plate 13.1 -> 12.2 ms.
-    if (n == 1 && team_size.size() == 1) {
-      const int sms = num_sms(), blocks = cmax(0);
-      const int per_sm = std::min(occ, (blocks + sms - 1) / sms);
-      const int c = std::min(std::max(blocks, b->slots[b->active[0]]->units), sms * per_sm);
-      used += std::max(0, c - team_size[0]);
-      team_size[0] = std::max(team_size[0], c);
-    }
     // the one-CTA instances are not bound to the bins the plan sized: they form a queue in decreasing work,
     // served by one-CTA workers (every CTA the multi-CTA teams leave, at least as many as the bins) and by the
     // CTAs of the multi-CTA teams once their instance is done, so that the estimates' errors even out
@@ -410,6 +400,24 @@ int rebuild_tables(shell_batch *b) {
       team_size.push_back(1);
       team_inst.push_back({});
       used += 1;
+    }
+    // An instance alone leaves SMs idle: phases that split into more units than row blocks (forces, the down step's
+    // residual and restriction blocks, the dense level's rows) get a CTA per unit, as far as the CTAs per SM that its
+    // row blocks take anyway reach (more would only lengthen the barriers). With the dense level's split among many
+    // CTAs (dense_level), per call: 24 x 17 panel in FP64 958 -> 737 us, 97 x 62 Jacobi case 780 -> 678 us, 128 x 128
+    // cylinder 4.33 -> 3.94 ms, in FP64 7.38 -> 6.15 ms, 512 x 512 plate 13.1 -> 12.2 ms. An instance of one row block
+    // keeps its one CTA, whose barriers cost nothing, unless it has a dense product to share out.
+    if (n == 1) {
+      const shell_handle *h = b->slots[b->active[0]];
+      const int sms = num_sms(), blocks = cmax(0);
+      const int per_sm = std::min(occ, (blocks + sms - 1) / sms);
+      const bool dense = h->h.amg_levels == 1 && h->h.amg_dense_n >= kDenseTeamRows;
+      const int c = blocks == 1 && !dense ? 1 : std::min(std::max(blocks, h->units), sms * per_sm);
+      team_of[0] = 0;
+      team_size = {std::max(c, team_size.empty() || !queue.empty() ? 1 : team_size[0])};
+      team_inst = {{0}};
+      queue.clear();
+      used = team_size[0];
     }
   }
   if (CS) {
@@ -868,6 +876,74 @@ std::vector<double> to_soa(const double *aos, int nv) {
 // projected system has removed; the doubled diagonal ties the constrained vertices down instead. Level 0 then
 // carries that matrix's values, and the instance's inverse diagonal (Jacobi, and the level-0 pre-smoothing
 // done in the residual and update phases) becomes its own, so the cycle stays symmetric.
+// Small meshes: the inverse of the step matrix as the preconditioner, one dense product in place of a multigrid cycle or
+// of Jacobi's many iterations. It replaces 7 to 15 iterations of six phases each by one or two of three, so it pays
+// until one CTA's read of the inverse (4 n^2 bytes from L2, 16 k clocks at n = 512) costs as much as those iterations;
+// the limit lies there because the set-up (7 ms of one host core at n = 529, 2 ms at 289) grows with n^2 times the
+// band. Per call: 289-vertex plate 343 -> 159 us, 450-vertex panel in FP64 740 -> 125 us, 24 FP64 instances of 81 to
+// 4,225 vertices 3.05 -> 2.64 ms, batch of 256 31.4 -> 31.0 ms. Leaves amg_levels at 0 where the inverse cannot be held in the solve's precision (see band_inverse).
+constexpr int kDenseRows = 512;
+int setup_dense(shell_handle *h, const HostCsr &A, const HostTopo &T) {
+  Inst &I = h->h;
+  cudaStream_t st = h->mem.st;
+  const int nv = I.nv;
+  if (nv > kDenseRows) return SHELL_OK;
+  std::vector<uint8_t> skip(nv, 1);   // rows coupled to no other (pinned vertices)
+  for (int i = 0; i < nv; ++i)
+    for (int k = A.ptr[i]; k < A.ptr[i + 1]; ++k)
+      if (A.col[k] != i && A.val[k] != 0.0) skip[i] = 0;
+  std::vector<int32_t> perm;
+  const int band = band_order(T, skip.data(), &perm);
+  const bool wide = I.precision == SHELL_FP64;
+  std::vector<double> inv;
+  if (!band_inverse(A, perm, band, wide ? 0x1p-53 : 0x1p-24, &inv)) return SHELL_OK;
+  AmgDev D{};
+  AmgDev *d_lev = nullptr;
+  double *inv64 = nullptr;
+  float *inv32 = nullptr;
+  auto layout = [&](Carver &C) {
+    D.b = C.take<double>(4 * (size_t)nv);
+    D.x = C.take<double>(4 * (size_t)nv);
+    if (wide)
+      inv64 = C.take<double>(inv.size());
+    else
+      inv32 = C.take<float>(inv.size());
+    d_lev = C.take<AmgDev>(1);
+  };
+  Carver sz;
+  layout(sz);
+  h->amg_bytes = sz.off;
+  h->amg_block = h->mem.get(h->amg_bytes);
+  if (!h->amg_block) return SHELL_ERR_OOM;
+  Carver real;
+  real.base = (char *)h->amg_block;
+  layout(real);
+  D.n = nv;
+  D.dinv32 = I.dinv32;
+  D.dinv64 = I.dinv64;
+  std::vector<float> narrow;
+  if (!wide) narrow.assign(inv.begin(), inv.end());
+  CK(cudaMemsetAsync(D.b, 0, 32 * (size_t)nv, st));
+  CK(cudaMemsetAsync(D.x, 0, 32 * (size_t)nv, st));
+  if (wide)
+    CK(cudaMemcpyAsync(inv64, inv.data(), 8 * inv.size(), cudaMemcpyHostToDevice, st));
+  else
+    CK(cudaMemcpyAsync(inv32, narrow.data(), 4 * narrow.size(), cudaMemcpyHostToDevice, st));
+  CK(cudaMemcpyAsync(d_lev, &D, sizeof(AmgDev), cudaMemcpyHostToDevice, st));
+  h->vcycle_bytes = 4 * (int64_t)inv.size() + 32 * (int64_t)nv;
+  if (nv >= kDenseTeamRows) h->units = std::max(h->units, (nv + 7) / 8);
+  I.amg_levels = 1;
+  I.amg_coarse_n = nv;
+  I.amg_dense_level = 0;
+  I.amg_dense_n = nv;
+  I.amg_dense64 = inv64;
+  I.amg_dense32 = inv32;
+  I.amg = d_lev;
+  CK(cudaMemcpyAsync(h->d_inst, &I, sizeof(Inst), cudaMemcpyHostToDevice, st));
+  CK(cudaStreamSynchronize(st));   // the host vectors go out of scope
+  return SHELL_OK;
+}
+
 int setup_amg(shell_handle *h, const HostTopo &T, int mode, bool stage, const std::vector<uint8_t> &fixb) {
   Inst &I = h->h;
   cudaStream_t st = h->mem.st;
@@ -895,7 +971,7 @@ int setup_amg(shell_handle *h, const HostTopo &T, int mode, bool stage, const st
     if (mass[r] > 0 && T.row_ptr[r + 1] - T.row_ptr[r] > 1) q.push_back((d - mass[r]) / mass[r]);
   }
   if (mode == SHELL_PRECOND_AUTO) {
-    if (nv < 256 || q.empty()) return SHELL_OK;
+    if (q.empty()) return SHELL_OK;
     std::nth_element(q.begin(), q.begin() + q.size() / 2, q.end());
     if (q[q.size() / 2] <= 30.0) return SHELL_OK;
   }
@@ -906,6 +982,11 @@ int setup_amg(shell_handle *h, const HostTopo &T, int mode, bool stage, const st
       if (A.col[k] == r) A.val[k] *= 2.0;
     val[T.diag_pos[r]] *= 2.0;
     own0 = true;
+  }
+  if (mode == SHELL_PRECOND_AUTO) {
+    const int rc = setup_dense(h, A, T);
+    if (rc != SHELL_OK || I.amg_levels > 0) return rc;
+    if (nv < 256) return SHELL_OK;
   }
   HostAmg H;
   build_amg(A, &H);

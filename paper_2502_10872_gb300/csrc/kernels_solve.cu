@@ -1434,13 +1434,16 @@ __device__ bool up_step(const Inst &I, int l, const Team &tm) {
 // large team) gives each row four lanes of every warp, one part each; otherwise a lane takes a row and the four parts
 // in turn. (A lane per row throughout left 26 of 32 lanes idle where 66 CTAs share 351 rows: 7.2 k clocks, and in
 // FP64, where an instruction costs the pipe 16 clocks for any number of active lanes, 25 k.)
-template <typename R>
+// Level 0 (a small mesh, whose whole preconditioner is the dense inverse): the output is u (in g), projected like
+// up_step's.
+template <typename R, bool MK>
 __device__ bool dense_level(const Inst &I, const Team &tm) {
   typedef typename Vec<R>::G G;
   constexpr int U = 8;
   const AmgDev &D = I.amg[I.amg_dense_level];
   const G *b = reinterpret_cast<const G *>(D.b);
-  R *y = reinterpret_cast<R *>(D.y);
+  R *y = reinterpret_cast<R *>(I.amg_dense_level == 0 ? I.g : D.y);
+  const uint8_t *fix = (MK && I.amg_dense_level == 0) ? I.fix : nullptr;
   const R *B = LevelVal<R>::dense(I);
   const int n = I.amg_dense_n;
   const int per = (n + tm.size - 1) / tm.size;
@@ -1523,6 +1526,7 @@ __device__ bool dense_level(const Inst &I, const Team &tm) {
       R sum = part[lane][0][w];
 #pragma unroll
       for (int g = 1; g < kBlock / 32; ++g) sum += part[lane][g][w];
+      if (fix && ((fix[io] >> w) & 1)) sum = R(0);
       y[4 * io + w] = sum;
     }
     __syncthreads();
@@ -1538,10 +1542,10 @@ __device__ bool dense_level(const Inst &I, const Team &tm) {
 // right-hand side. Returns false on abort.
 template <typename R, bool MK = false>
 __device__ bool vcycle(const Inst &I, const Team &tm) {
-  const int top = I.amg_dense_level > 0 ? I.amg_dense_level : I.amg_levels - 1;
+  const int top = I.amg_dense_level >= 0 ? I.amg_dense_level : I.amg_levels - 1;   // 0: the dense inverse alone
   for (int l = 0; l < top; ++l)
     if (!down_step<R>(I, l, tm)) return false;
-  if (!(I.amg_dense_level > 0 ? dense_level<R>(I, tm) : coarsest<R>(I, tm))) return false;
+  if (!(I.amg_dense_level >= 0 ? dense_level<R, MK>(I, tm) : coarsest<R>(I, tm))) return false;
   for (int l = top - 1; l >= 0; --l)
     if (!up_step<R, MK>(I, l, tm)) return false;
   return true;
@@ -1778,7 +1782,8 @@ __device__ int cg_loop(const Inst &I, Team &tm, double *x, double tol2, int max_
     const CgScalars &S = cg_state();
     *rho_out = S.rho;
     if (S.verdict <= 0) return S.verdict == 0 ? it : S.verdict;
-    const bool look = direct || (S.look && I.amg_levels > 0);
+    // an inverse as the preconditioner converges at once: always worth the look
+    const bool look = direct || (I.amg_levels > 0 && (S.look || I.amg_levels == 1));
     phase_update<R>(I, tm, CgCoef<R>::alpha(S), CgCoef<R>::beta(S), it == 0, x, S.alpha, look, direct);
     if (!team_sync(tm)) return -2;
     if (look) {
