@@ -229,8 +229,6 @@ void destroy_graph(shell_batch *b) {
   b->graph_tried = false;
 }
 
-constexpr int kDenseTeamRows = 128;   // rows from which a dense inverse is worth a team of CTAs (four passes of one CTA)
-
 // The step kernel's variant with the Newton tangent also carries the projection of per-component constraints.
 static bool uses_nt_variant(const Inst &I) { return (I.nl_newton && I.nl_max > 1) || I.fix != nullptr; }
 
@@ -411,7 +409,7 @@ int rebuild_tables(shell_batch *b) {
       const shell_handle *h = b->slots[b->active[0]];
       const int sms = num_sms(), blocks = cmax(0);
       const int per_sm = std::min(occ, (blocks + sms - 1) / sms);
-      const bool dense = h->h.amg_levels == 1 && h->h.amg_dense_n >= kDenseTeamRows;
+      const bool dense = h->h.amg_levels == 1;
       const int c = blocks == 1 && !dense ? 1 : std::min(std::max(blocks, h->units), sms * per_sm);
       team_of[0] = 0;
       team_size = {std::max(c, team_size.empty() || !queue.empty() ? 1 : team_size[0])};
@@ -876,8 +874,8 @@ std::vector<double> to_soa(const double *aos, int nv) {
 // projected system has removed; the doubled diagonal ties the constrained vertices down instead. Level 0 then
 // carries that matrix's values, and the instance's inverse diagonal (Jacobi, and the level-0 pre-smoothing
 // done in the residual and update phases) becomes its own, so the cycle stays symmetric.
-// Small meshes: the inverse of the step matrix as the preconditioner, one dense product in place of a multigrid cycle or
-// of Jacobi's many iterations. It replaces 7 to 15 iterations of six phases each by one or two of three, so it pays
+// Small meshes: the inverse of the step matrix as the preconditioner, one dense product in place of a multigrid cycle
+// (and, like it, from 256 vertices on: below, callers that cap the iterations rely on Jacobi's). It replaces 7 to 15 iterations of six phases each by one or two of three, so it pays
 // until one CTA's read of the inverse (4 n^2 bytes from L2, 16 k clocks at n = 512) costs as much as those iterations;
 // the limit lies there because the set-up (7 ms of one host core at n = 529, 2 ms at 289) grows with n^2 times the
 // band. Per call: 289-vertex plate 343 -> 159 us, 450-vertex panel in FP64 740 -> 125 us, 24 FP64 instances of 81 to
@@ -931,7 +929,7 @@ int setup_dense(shell_handle *h, const HostCsr &A, const HostTopo &T) {
     CK(cudaMemcpyAsync(inv32, narrow.data(), 4 * narrow.size(), cudaMemcpyHostToDevice, st));
   CK(cudaMemcpyAsync(d_lev, &D, sizeof(AmgDev), cudaMemcpyHostToDevice, st));
   h->vcycle_bytes = 4 * (int64_t)inv.size() + 32 * (int64_t)nv;
-  if (nv >= kDenseTeamRows) h->units = std::max(h->units, (nv + 7) / 8);
+  h->units = std::max(h->units, (nv + 7) / 8);
   I.amg_levels = 1;
   I.amg_coarse_n = nv;
   I.amg_dense_level = 0;
@@ -971,7 +969,7 @@ int setup_amg(shell_handle *h, const HostTopo &T, int mode, bool stage, const st
     if (mass[r] > 0 && T.row_ptr[r + 1] - T.row_ptr[r] > 1) q.push_back((d - mass[r]) / mass[r]);
   }
   if (mode == SHELL_PRECOND_AUTO) {
-    if (q.empty()) return SHELL_OK;
+    if (nv < 256 || q.empty()) return SHELL_OK;
     std::nth_element(q.begin(), q.begin() + q.size() / 2, q.end());
     if (q[q.size() / 2] <= 30.0) return SHELL_OK;
   }
@@ -986,7 +984,6 @@ int setup_amg(shell_handle *h, const HostTopo &T, int mode, bool stage, const st
   if (mode == SHELL_PRECOND_AUTO) {
     const int rc = setup_dense(h, A, T);
     if (rc != SHELL_OK || I.amg_levels > 0) return rc;
-    if (nv < 256) return SHELL_OK;
   }
   HostAmg H;
   build_amg(A, &H);
