@@ -1259,9 +1259,11 @@ int shell_create(const shell_mesh *mesh, const shell_material *mat, int32_t mode
   I.precision = opt.precision;
   I.kt = T.kt;
   I.n_slices = T.n_slices;
-  I.rows_per_thread = 1;
-  const int chunk = kBlock * I.rows_per_thread;
-  I.n_chunks = (nv + chunk - 1) / chunk;
+  // FP64 instances split into chunks of down to a warp's rows, at most about one per SM (see row_threads)
+  I.chunk_rows = kBlock;
+  if (I.precision == SHELL_FP64)
+    for (I.chunk_rows = 32; I.chunk_rows < kBlock && nv > 152 * I.chunk_rows;) I.chunk_rows *= 2;
+  I.n_chunks = (nv + I.chunk_rows - 1) / I.chunk_rows;
   I.pcg_max_it = opt.pcg_max_it;
   I.refine_max = opt.refine_max;
   I.nl_max = 0;        // linearised step until shell_set_nonlinear
@@ -1273,7 +1275,8 @@ int shell_create(const shell_mesh *mesh, const shell_material *mat, int32_t mode
   I.lam = mat->E * mat->nu / (1.0 - mat->nu * mat->nu);
   I.n_slots = T.n_slots;
   I.n_local = T.n_local;
-  if (I.precision != SHELL_FP64) h->units = (nt + T.ne + kBlock - 1) / kBlock;   // forces in the step kernel
+  h->units = I.precision == SHELL_FP64 ? (nv + 31) / 32                         // level 0 in passes of a warp's rows
+                                       : (nt + T.ne + kBlock - 1) / kBlock;     // forces in the step kernel
   const size_t nnz_pad = (size_t)T.sl_ptr[T.n_slices];
   h->nnz = T.nnz;
   h->nnz_pad = (int64_t)nnz_pad;
@@ -1293,10 +1296,13 @@ int shell_create(const shell_mesh *mesh, const shell_material *mat, int32_t mode
     std::vector<uint8_t> skip(nv);
     for (int i = 0; i < nv; ++i) skip[i] = fixb[i] == 7;
     const int w = (3 * band_order(T, skip.data(), &perm) + 2) | 1;   // odd: column reads without bank conflicts
-    if ((size_t)3 * nv * (w + 3) <= (size_t)kDirectWords)
+    if ((size_t)3 * nv * (w + 3) <= (size_t)kDirectWords) {
       I.dir_w = w;
-    else
+      I.chunk_rows = kBlock;   // factored and solved by one CTA: no team
+      I.n_chunks = 1;
+    } else {
       perm.clear();
+    }
   }
 
   // ---- persistent block

@@ -92,7 +92,7 @@ struct Inst {
   int32_t precision;             // shell_precision
   int32_t kt;                    // contribution slots per triangle: 6 (triangle stencils) or 3 (membrane only)
   int32_t n_slices;              // SELL slices
-  int32_t rows_per_thread;       // rows per thread of a reduction chunk (chunk = kBlock * rows_per_thread)
+  int32_t chunk_rows;            // rows of a reduction chunk: kBlock, FP64 also 32, 64 or 128
   int32_t n_chunks;
   int32_t pcg_max_it, refine_max;
   int32_t nl_max;                // chord iterations per step of the exact backward Euler (<= 1: linearised step)

@@ -10,8 +10,8 @@
 // FP32 products stage each block's gathered vector entries in shared memory (per-block gather lists).
 //
 // Work split. The grid is cut into teams of CTAs; a team processes a fixed list of instances one after the
-// other, all of its CTAs working on the same instance. Rows are grouped in chunks of kBlock * rpt rows
-// (rpt = rows per thread, fixed per instance); chunk c is owned by team rank c mod team_size. Teams of one
+// other, all of its CTAs working on the same instance. Row block k belongs to team rank k mod team_size (see
+// row_threads); sums are formed over chunks of chunk_rows rows, fixed per instance. Teams of one
 // CTA synchronise with __syncthreads; larger teams with a global-memory barrier whose spin is bounded in
 // time (on timeout the kernel raises an abort flag and every CTA returns). The launch is cooperative, so
 // all CTAs are co-resident and the barrier cannot wait for a CTA that is not running.
@@ -62,6 +62,7 @@ struct Team {
   unsigned long long t0;   // start of the current instance's solve (global timer, ns)
   int cap;      // vector entries the dynamic shared memory can stage (0: no staging)
   int chord_k;  // chord iteration of the step this launch performs
+  int act;      // threads of a CTA that take rows of the current instance (see row_threads)
   unsigned long long wait_ns;   // bound of a barrier wait
 };
 
@@ -162,14 +163,42 @@ __device__ __forceinline__ double octet_sum(double v) {
   return v;
 }
 
-// Per-chunk partials: each chunk's three values are reduced by a fixed tree (warp shuffles, then the warps'
-// sums). The warp sums of up to kStage chunks are staged in shared memory and written out together, so
-// a CTA that owns several chunks of a phase pays two __syncthreads per kStage chunks instead of per chunk.
+// Row blocks. A pass of a CTA takes `act` consecutive rows, a thread each (the other threads idle), block k of an
+// instance going to team rank k mod size. FP32 instances always take kBlock rows, which their gather lists are made
+// for. FP64 instances are bound by the FP64 pipe (a warp instruction occupies it for 16 clocks, so a product of 256
+// rows with 19 entries takes 7.3 k clocks of one SM), so their passes shrink down to a warp's rows while that gives
+// more CTAs of the team a block: 128 x 128 cylinder in FP64 6.14 -> 5.60 ms a call of 4 steps, 24 FP64 instances of 81 to
+// 4,225 vertices 2.56 -> 1.52 ms. Which CTA computes a row does not change its value.
+// units(log): blocks of a phase at passes of 2^log threads. Returns the log.
+constexpr int kBlockLog = 8;
+static_assert(1 << kBlockLog == kBlock, "log of the CTA's threads");
+template <typename F>
+__device__ __forceinline__ int fewest_threads_log(int size, F units) {
+  int log = kBlockLog;
+  while (log > 5 && units(log - 1) <= size) --log;
+  return log;
+}
+__device__ __forceinline__ int blocks_of(int n, int log) { return (n + (1 << log) - 1) >> log; }
+template <typename R>
+__device__ __forceinline__ int level_threads(int n, const Team &tm) {
+  if (sizeof(R) == 4) return kBlock;
+  return 1 << fewest_threads_log(tm.size, [&](int log) { return blocks_of(n, log); });
+}
+// of the phases with sums: whole chunks
+__device__ inline int row_threads(const Inst &I, int size) {
+  if (I.precision != SHELL_FP64) return kBlock;
+  const int nv = I.nv;
+  return max(I.chunk_rows, 1 << fewest_threads_log(size, [&](int log) { return blocks_of(nv, log); }));
+}
+
+// Per-chunk partials: each chunk's (chunk_rows rows') three values are reduced by a fixed tree (warp shuffles, then the
+// warps' sums). The warp sums of up to kStage passes are staged in shared memory and written out together, so
+// a CTA that makes several passes in a phase pays two __syncthreads per kStage passes instead of per pass.
 constexpr int kStage = 32;
 
 struct ChunkStage {
-  int n = 0;       // staged chunks
-  int first = 0;   // chunk id of the first staged one
+  int n = 0;       // staged passes
+  int first = 0;   // block of the first staged one
 };
 
 __device__ inline double (*stage_buf())[kBlock / 32][3] {
@@ -178,28 +207,34 @@ __device__ inline double (*stage_buf())[kBlock / 32][3] {
 }
 
 // A: the type the warp sums were staged in (FP32 sums are widened here: 24 lanes of one warp instead of one lane of
-// each warp and value)
+// each warp and value). Lane 8 k + w holds warp w's sum of value k; the warps of a chunk are added by a tree.
 template <typename A>
 __device__ void stage_flush(ChunkStage &cs, const Inst &I, const Team &tm) {
   const A(*sm)[kBlock / 32][3] = reinterpret_cast<const A(*)[kBlock / 32][3]>(stage_buf());
-  const int lane = threadIdx.x & 31;
+  const int lane = threadIdx.x & 31, w = lane & 7;
+  const int act = tm.act, per = I.chunk_rows >> 5;   // warps per chunk
+  const int log = 31 - __clz(I.chunk_rows);
   __syncthreads();
-  for (int k = threadIdx.x >> 5; k < cs.n; k += kBlock / 32) {   // a warp per chunk
-    double v = lane < 24 ? double(sm[k][lane & 7][lane >> 3]) : 0.0;
-    v = octet_sum(v);
-    if ((lane & 7) == 0 && lane < 24) part_of(I, tm, cs.first + k * tm.size)[lane >> 3] = v;
+  for (int k = threadIdx.x >> 5; k < cs.n; k += kBlock / 32) {   // a warp per pass
+    const bool in = lane < 24 && 32 * w < act;
+    double v = in ? double(sm[k][w][lane >> 3]) : 0.0;
+    for (int o = per / 2; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    const int ch = ((cs.first + k * tm.size) * act + 32 * w) >> log;
+    if (in && (w & (per - 1)) == 0 && ch < I.n_chunks) part_of(I, tm, ch)[lane >> 3] = v;
   }
   __syncthreads();
   cs.n = 0;
 }
 
 template <typename A>
-__device__ void stage_chunk(ChunkStage &cs, const Inst &I, const Team &tm, int ch, A v0, A v1, A v2) {
+__device__ void stage_chunk(ChunkStage &cs, const Inst &I, const Team &tm, int blk, A v0, A v1, A v2) {
   A(*sm)[kBlock / 32][3] = reinterpret_cast<A(*)[kBlock / 32][3]>(stage_buf());
-  if (cs.n == 0) cs.first = ch;
+  if (cs.n == 0) cs.first = blk;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const A v = warp_sum3(v0, v1, v2);
-  if ((lane & 7) == 0 && lane < 24) sm[cs.n][warp][lane >> 3] = v;
+  if (32 * warp < tm.act) {
+    const A v = warp_sum3(v0, v1, v2);
+    if ((lane & 7) == 0 && lane < 24) sm[cs.n][warp][lane >> 3] = v;
+  }
   if (++cs.n == kStage) stage_flush<A>(cs, I, tm);
 }
 
@@ -615,12 +650,10 @@ __device__ void phase_forces(const Inst &I, const Team &tm) {
 }
 
 #define ROWS_BEGIN(I, tm)                                                                 \
-  for (int ch = (tm).rank; ch < (I).n_chunks; ch += (tm).size) {                        \
-    for (int rr = 0; rr < (I).rows_per_thread; ++rr) {                                  \
-      const int row = (ch * (I).rows_per_thread + rr) * kBlock + (int)threadIdx.x;      \
-      if (row < (I).nv) {
+  for (int blk = (tm).rank; blk * (tm).act < (I).nv; blk += (tm).size) {                \
+    const int row = blk * (tm).act + (int)threadIdx.x;                                  \
+    if ((int)threadIdx.x < (tm).act && row < (I).nv) {
 #define ROWS_END \
-  }              \
   }              \
   }
 
@@ -644,11 +677,11 @@ __device__ inline int guess_order(const double e[3]) {
 __device__ void phase_history(const Inst &I, const Team &tm) {
   const int nv = I.nv;
   ChunkStage cs;
-  for (int ch = tm.rank; ch < I.n_chunks; ch += tm.size) {
+  const int act = tm.act;
+  for (int blk = tm.rank; blk * act < nv; blk += tm.size) {
     double e0 = 0.0, e1 = 0.0, e2 = 0.0;
-    for (int rr = 0; rr < I.rows_per_thread; ++rr) {
-      const int row = (ch * I.rows_per_thread + rr) * kBlock + (int)threadIdx.x;
-      if (row >= nv || ((threadIdx.x >> 5) + ch) % 4 != 0 || I.pinned[row]) continue;
+    const int row = blk * act + (int)threadIdx.x, w = row >> 5;
+    if ((int)threadIdx.x < act && row < nv && (w + w / (kBlock / 32)) % 4 == 0 && !I.pinned[row]) {
 #pragma unroll
       for (int c = 0; c < 3; ++c) {
         const int k = c * nv + row;
@@ -660,7 +693,7 @@ __device__ void phase_history(const Inst &I, const Team &tm) {
         e2 += d2 * d2;
       }
     }
-    stage_chunk<double>(cs, I, tm, ch, e0, e1, e2);
+    stage_chunk<double>(cs, I, tm, blk, e0, e1, e2);
   }
   if (cs.n) stage_flush<double>(cs, I, tm);
 }
@@ -699,11 +732,11 @@ __device__ void phase_rhs(const Inst &I, const Team &tm, int order) {
   const bool chord = tm.chord_k > 0;
   const RC *con = reinterpret_cast<const RC *>(I.contrib);
   ChunkStage cs;
-  for (int ch = tm.rank; ch < I.n_chunks; ch += tm.size) {
+  const int act = tm.act;
+  for (int blk = tm.rank; blk * act < nv; blk += tm.size) {
     double bb = 0.0;
-    for (int rr = 0; rr < I.rows_per_thread; ++rr) {
-      const int row = (ch * I.rows_per_thread + rr) * kBlock + (int)threadIdx.x;
-      if (row >= nv) continue;
+    const int row = blk * act + (int)threadIdx.x;
+    if ((int)threadIdx.x < act && row < nv) {
       ContribSum<RC> fs[3];
       // the vertex's slots in their fixed order, four per round: the slot indices, then their contributions
       // (written by the team's force phase: coherent loads), are in flight together
@@ -771,7 +804,7 @@ __device__ void phase_rhs(const Inst &I, const Team &tm, int order) {
       }
       if (!chord) reinterpret_cast<D4 *>(I.g64)[row] = {sv[0], sv[1], sv[2], 0.0};
     }
-    stage_chunk<double>(cs, I, tm, ch, bb, 0.0, 0.0);
+    stage_chunk<double>(cs, I, tm, blk, bb, 0.0, 0.0);
   }
   if (cs.n) stage_flush<double>(cs, I, tm);
 }
@@ -793,12 +826,11 @@ __device__ void phase_resid(const Inst &I, const Team &tm) {
   const R *dinv = Vec<R>::dinv(I);
   const bool st = I.h0.max > 0 && 2 * I.h0.max <= tm.cap;   // FP64 entries take two buffer slots
   ChunkStage cs;
-  for (int ch = tm.rank; ch < I.n_chunks; ch += tm.size) {
+  const int act = tm.act;
+  for (int blk = tm.rank; blk * act < nv; blk += tm.size) {
     double rr2 = 0.0;
-    for (int rr = 0; rr < I.rows_per_thread; ++rr) {
-      const int blk = ch * I.rows_per_thread + rr;
-      if (blk * kBlock >= nv) break;
-      const int row = blk * kBlock + (int)threadIdx.x;
+    do {   // this thread's row
+      const int row = (int)threadIdx.x < act ? blk * act + (int)threadIdx.x : nv;
       double ax, ay, az;
       if (st) {
         staged_row64(I.h0, blk, g64, I.sl_ptr, I.val64, row, row < nv, ax, ay, az);
@@ -845,8 +877,8 @@ __device__ void phase_resid(const Inst &I, const Team &tm) {
         const R d = om0 * di;
         x0[row] = Vec<R>::mk(d * q0, d * q1, d * q2);
       }
-    }
-    stage_chunk<double>(cs, I, tm, ch, rr2, 0.0, 0.0);
+    } while (false);
+    stage_chunk<double>(cs, I, tm, blk, rr2, 0.0, 0.0);
   }
   if (cs.n) stage_flush<double>(cs, I, tm);
 }
@@ -862,14 +894,13 @@ __device__ void phase_spmv(const Inst &I, const Team &tm) {
   bool st = false;
   if constexpr (sizeof(R) == 4) st = halo_on(I.h0, tm.cap);
   ChunkStage cs;
-  for (int ch = tm.rank; ch < I.n_chunks; ch += tm.size) {
+  const int act = tm.act;
+  for (int blk = tm.rank; blk * act < nv; blk += tm.size) {
     R gu = R(0), wu = R(0), rr2 = R(0);
-    for (int rr = 0; rr < I.rows_per_thread; ++rr) {
-      const int blk = ch * I.rows_per_thread + rr;
-      if (blk * kBlock >= nv) break;
+    do {   // this thread's row
       R ax, ay, az;
       typename Vec<R>::G u;
-      const int row = blk * kBlock + (int)threadIdx.x;
+      const int row = (int)threadIdx.x < act ? blk * act + (int)threadIdx.x : nv;
       R r0 = R(0), r1 = R(0), r2 = R(0);   // loaded before the product, whose latency hides theirs
       if (row < nv) {
         r0 = r[row];
@@ -911,8 +942,8 @@ __device__ void phase_spmv(const Inst &I, const Team &tm) {
       gu += r0 * R(u.x) + r1 * R(u.y) + r2 * R(u.z);
       wu += ax * R(u.x) + ay * R(u.y) + az * R(u.z);
       rr2 += r0 * r0 + r1 * r1 + r2 * r2;
-    }
-    stage_chunk<R>(cs, I, tm, ch, gu, wu, rr2);
+    } while (false);
+    stage_chunk<R>(cs, I, tm, blk, gu, wu, rr2);
   }
   if (cs.n) stage_flush<R>(cs, I, tm);
 }
@@ -943,11 +974,11 @@ __device__ void phase_update(const Inst &I, const Team &tm, R alpha, R beta, boo
   typename Vec<R>::G *x0 = amg ? reinterpret_cast<typename Vec<R>::G *>(I.amg[0].x) : nullptr;
   const R om0 = amg ? LevelVal<R>::omega(I.amg[0]) : R(0);
   ChunkStage cs;
-  for (int ch = tm.rank; ch < I.n_chunks; ch += tm.size) {
+  const int act = tm.act;
+  for (int blk = tm.rank; blk * act < nv; blk += tm.size) {
     R rr2 = R(0);
-    for (int rr = 0; rr < I.rows_per_thread; ++rr) {
-      const int row = (ch * I.rows_per_thread + rr) * kBlock + (int)threadIdx.x;
-      if (row >= nv) break;
+    const int row = blk * act + (int)threadIdx.x;
+    if ((int)threadIdx.x < act && row < nv) {
       const R di = dinv[row];
       // all loads before the first store: the stores may alias the next component's loads for all the compiler knows
       R uo[3], ro[3], po[3], so[3], wo[3];
@@ -992,7 +1023,7 @@ __device__ void phase_update(const Inst &I, const Team &tm, R alpha, R beta, boo
       }
       if (sum) rr2 += rv[0] * rv[0] + rv[1] * rv[1] + rv[2] * rv[2];
     }
-    if (sum) stage_chunk<R>(cs, I, tm, ch, R(0), R(0), rr2);
+    if (sum) stage_chunk<R>(cs, I, tm, blk, R(0), R(0), rr2);
   }
   if (cs.n) stage_flush<R>(cs, I, tm);
 }
@@ -1086,12 +1117,13 @@ __device__ inline void level_a(const AmgDev &L, const D4 *v, int row, double &ax
 
 // residual of one 256-row block of level 0: r = b - A x
 template <typename R, bool ST>
-__device__ __forceinline__ void resid_blk(const AmgDev &A, int blk) {
+__device__ __forceinline__ void resid_blk(const AmgDev &A, int blk, int act) {
   typedef typename Vec<R>::G G;
   const G *b = reinterpret_cast<const G *>(A.b);
   const G *x = reinterpret_cast<const G *>(A.x);
   G *rr = reinterpret_cast<G *>(A.r);
-  const int row = blk * kBlock + (int)threadIdx.x;
+  if ((int)threadIdx.x >= act) return;   // FP32: none
+  const int row = blk * act + (int)threadIdx.x;
   R ax, ay, az;
   if constexpr (ST) {
     float4 ui;
@@ -1111,10 +1143,10 @@ __device__ __forceinline__ void resid_blk(const AmgDev &A, int blk) {
 // (FP32) and unstaged products run the same arithmetic. The loads that do not depend on the staged vector
 // (slice bounds, first nonzeros) are issued before the staging barrier.
 template <typename R, bool ST>
-__device__ __forceinline__ void restrict_blk(const AmgDev &A, const AmgDev &C, bool pre, int blk) {
+__device__ __forceinline__ void restrict_blk(const AmgDev &A, const AmgDev &C, bool pre, int blk, int act) {
   typedef typename Vec<R>::G G;
   constexpr int U = 8;
-  constexpr int kRows = kBlock / 4;   // coarse rows per CTA pass
+  if ((int)threadIdx.x >= act) return;   // whole warps
   const G *bf = reinterpret_cast<const G *>(A.b);
   G *bc = reinterpret_cast<G *>(C.b);
   G *xc = reinterpret_cast<G *>(C.x);
@@ -1123,7 +1155,7 @@ __device__ __forceinline__ void restrict_blk(const AmgDev &A, const AmgDev &C, b
   const R omc = LevelVal<R>::omega(C);
   const int n = A.n_next;
   const int lane = threadIdx.x & 31;
-  const int row = blk * kRows + (int)(threadIdx.x >> 2);
+  const int row = blk * (act / 4) + (int)(threadIdx.x >> 2);
   const bool valid = row < n;
   int p = 0, b1 = 0;
   if (valid) {
@@ -1193,8 +1225,10 @@ __device__ void lv_up(const AmgDev &A, const AmgDev &C, typename Vec<R>::G *y, c
   const G *yc = reinterpret_cast<const G *>(C.y);
   const R *dinv = LevelVal<R>::dinv(A);
   const R om = LevelVal<R>::omega(A);
-  for (int ch = tm.rank; ch * kBlock < A.n; ch += tm.size) {
-    const int row = ch * kBlock + (int)threadIdx.x;
+  const int act = level_threads<R>(A.n, tm);
+  for (int ch = tm.rank; ch * act < A.n; ch += tm.size) {
+    if ((int)threadIdx.x >= act) continue;   // FP32: none
+    const int row = ch * act + (int)threadIdx.x;
     R ax, ay, az;
     if constexpr (ST) {
       float4 unused;
@@ -1307,12 +1341,13 @@ __device__ __forceinline__ void coarse_row(const AmgDev &A, const typename Vec<R
 
 // residual of one 64-row block of a coarse level: r = b - A x
 template <typename R, bool ST>
-__device__ __forceinline__ void resid4_blk(const AmgDev &A, int blk) {
+__device__ __forceinline__ void resid4_blk(const AmgDev &A, int blk, int act) {
   typedef typename Vec<R>::G G;
   const G *b = reinterpret_cast<const G *>(A.b);
   const G *x = reinterpret_cast<const G *>(A.x);
   G *rr = reinterpret_cast<G *>(A.r);
-  const int row = blk * (kBlock / 4) + (int)(threadIdx.x >> 2);
+  if ((int)threadIdx.x >= act) return;   // whole warps
+  const int row = blk * (act / 4) + (int)(threadIdx.x >> 2);
   const bool valid = row < A.n;
   R ax, ay, az;
   G ui;
@@ -1360,28 +1395,31 @@ __device__ bool down_step(const Inst &I, int l, const Team &tm) {
   // levels at and below the dense level, and the coarsest, are solved, not smoothed
   const int top = I.amg_dense_level > 0 ? I.amg_dense_level : I.amg_levels - 1;
   const bool pre = l + 1 < top;
-  const int fr = l == 0 ? kBlock : kBlock / 4;   // rows per residual block
-  const int nf = (A.n + fr - 1) / fr;
-  const int nu = nf + (A.n_next + kBlock / 4 - 1) / (kBlock / 4);
+  // residual blocks of act rows (4 threads a row on the coarse levels) and restriction blocks of act / 4 rows
+  const int n = A.n, nn = A.n_next;
+  auto resids = [&](int log) { return blocks_of(n, l == 0 ? log : log - 2); };
+  auto units = [&](int log) { return resids(log) + blocks_of(nn, log - 2); };
+  const int log = sizeof(R) == 4 ? kBlockLog : fewest_threads_log(tm.size, units);
+  const int act = 1 << log, nf = resids(log), nu = units(log);
   const bool sa = staged<R>(A.ha, tm.cap), sr = staged<R>(A.hr, tm.cap);
   for (int u = tm.rank; u < nu; u += tm.size) {
     if (u < nf) {
       if (l == 0) {
         if (sa)
-          resid_blk<R, (sizeof(R) == 4)>(A, u);
+          resid_blk<R, (sizeof(R) == 4)>(A, u, act);
         else
-          resid_blk<R, false>(A, u);
+          resid_blk<R, false>(A, u, act);
       } else {
         if (sa)
-          resid4_blk<R, (sizeof(R) == 4)>(A, u);
+          resid4_blk<R, (sizeof(R) == 4)>(A, u, act);
         else
-          resid4_blk<R, false>(A, u);
+          resid4_blk<R, false>(A, u, act);
       }
     } else {
       if (sr)
-        restrict_blk<R, (sizeof(R) == 4)>(A, C, pre, u - nf);
+        restrict_blk<R, (sizeof(R) == 4)>(A, C, pre, u - nf, act);
       else
-        restrict_blk<R, false>(A, C, pre, u - nf);
+        restrict_blk<R, false>(A, C, pre, u - nf, act);
     }
   }
   return team_sync(tm);
@@ -1871,11 +1909,11 @@ __device__ bool team_max_step(const Inst &I, Team &tm, double *out) {
   __shared__ double res;
   const int nv = I.nv, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const bool first = tm.chord_k == 0;
-  for (int ch = tm.rank; ch < I.n_chunks; ch += tm.size) {
+  const int act = tm.act, per = act / I.chunk_rows;   // chunks of a pass: each gets the pass's maximum
+  for (int blk = tm.rank; blk * act < nv; blk += tm.size) {
     double mx = 0.0;
-    for (int rr = 0; rr < I.rows_per_thread; ++rr) {
-      const int row = (ch * I.rows_per_thread + rr) * kBlock + (int)threadIdx.x;
-      if (row >= nv) continue;
+    const int row = blk * act + (int)threadIdx.x;
+    if ((int)threadIdx.x < act && row < nv) {
       for (int c = 0; c < 3; ++c) {
         const int k = c * nv + row;
         mx = fmax(mx, fabs(I.sol[k] - (first ? 0.0 : I.vk[k])));
@@ -1888,7 +1926,7 @@ __device__ bool team_max_step(const Inst &I, Team &tm, double *out) {
     if (threadIdx.x == 0) {
       double m = wmax[0];
       for (int w = 1; w < kBlock / 32; ++w) m = fmax(m, wmax[w]);
-      part_of(I, tm, ch)[0] = m;
+      for (int ch = blk * per; ch < min((blk + 1) * per, I.n_chunks); ++ch) part_of(I, tm, ch)[0] = m;
     }
     __syncthreads();
   }
@@ -2257,6 +2295,7 @@ __global__ void __launch_bounds__(kBlock, MINB) k_solve(const Inst *__restrict__
       tm.size = in_queue ? 1 : team_size;
       tm.rank = in_queue ? 0 : team_rank;
       tm.mode = in_queue ? 0 : team_mode;
+      tm.act = row_threads(I, tm.size);
       tm.t0 = gtimer();
     }
     __syncthreads();
