@@ -240,7 +240,7 @@ __device__ void stage_chunk(ChunkStage &cs, const Inst &I, const Team &tm, int b
 
 // sum all chunk partials of an instance in a fixed order; result broadcast to the CTA. Flips the bank, so
 // the next phase may write partials while slower CTAs of the team still read these.
-// then(sum): run by the thread that holds the sums, before they are broadcast.
+// then(sum): run by the warp that holds the sums, before they are broadcast.
 template <typename F>
 __device__ __forceinline__ void team_reduce(const Inst &I, Team &tm, double out[3], F then) {
   __shared__ double res[3];
@@ -276,10 +276,8 @@ __device__ __forceinline__ void team_reduce(const Inst &I, Team &tm, double out[
   if (warp == 0) {
     if ((lane & 7) == 0 && lane < 24) res[lane >> 3] = v;
     __syncwarp();
-    if (lane == 0) {
-      tm.bank ^= 1;   // the partials' readers of this CTA have read theirs
-      then(res);
-    }
+    if (lane == 0) tm.bank ^= 1;   // the partials' readers of this CTA have read theirs
+    then(res);
   }
   __syncthreads();
   out[0] = res[0];
@@ -1755,7 +1753,7 @@ __device__ __noinline__ void direct_apply(const Inst &I) {
   if (v < nv) g[v] = {y[p], y[p + 1], y[p + 2], 0.0};
 }
 
-// Scalars of the recurrence, computed by one thread of the CTA from the reduced sums and read by the others from
+// Scalars of the recurrence, computed by one warp of the CTA from the reduced sums and read by the others from
 // shared memory: three dependent FP64 divisions in every thread occupied the FP64 pipe (2 operations per clock and
 // SM on GB300) for several thousand clocks of each iteration. Per call, with the smoother's weight read in FP32
 // instead of converted by every thread in every phase: 512 x 512 plate 19.0 -> 18.2 ms (4 steps), 128 x 128 cylinder
@@ -1788,11 +1786,25 @@ struct CgCoef<double> {
 // residual is summed right away (one more reduction) and a converged solve ends there: the same test on the same sums.
 // The margin is wide (a factor 5 of the norm): a look in vain costs a reduction, a missed one a V-cycle and a product.
 constexpr double kLookAhead = 25.0;
+// The warp that reduced the sums calls it: three lanes share one division's latency (several hundred clocks in FP64) for
+// beta, gamma' / alpha and the reduction rate, and the division for alpha' follows; one thread doing the four in turn took
+// half of a reduction's 4.2 k clocks.
 template <typename R>
 __device__ inline void cg_scalars(const double *sum, int it, double tol2, int max_it) {
   CgScalars &s = cg_state();
+  const int lane = threadIdx.x & 31;
   const double gn = sum[0], dn = sum[1], rho = sum[2];
-  if (it > 0) s.rate = rho / s.rho;
+  double bn = 0.0, pole = 0.0, rate = 0.0;
+  if (it > 0) {
+    const double q = (lane == 2 ? rho : gn) / (lane == 0 ? s.gamma : lane == 1 ? s.alpha : s.rho);
+    bn = __shfl_sync(0xffffffffu, q, 0);
+    pole = bn * __shfl_sync(0xffffffffu, q, 1);
+    rate = __shfl_sync(0xffffffffu, q, 2);
+  }
+  const double alpha = gn / (dn - pole);
+  __syncwarp();
+  if (lane != 0) return;
+  if (it > 0) s.rate = rate;
   s.rho = rho;
   s.look = rho * s.rate <= kLookAhead * tol2;
   if (!isfinite(rho) || !isfinite(gn) || !isfinite(dn)) {
@@ -1802,11 +1814,10 @@ __device__ inline void cg_scalars(const double *sum, int it, double tol2, int ma
   } else if (it >= max_it) {
     s.verdict = -1;
   } else {
-    const double bn = it == 0 ? 0.0 : gn / s.gamma;
-    s.alpha = it == 0 ? gn / dn : gn / (dn - bn * gn / s.alpha);
+    s.alpha = alpha;
     s.beta = bn;
     s.gamma = gn;
-    s.alpha32 = float(s.alpha);
+    s.alpha32 = float(alpha);
     s.beta32 = float(bn);
     s.verdict = 1;
   }
