@@ -268,8 +268,9 @@ int rebuild_tables(shell_batch *b) {
   // a batch with a Newton instance, or one with per-component constraints, runs the variant that carries the
   // Newton tangent and the projection
   b->prec = anynt ? 3 : (any64 && any32) ? 0 : (any64 ? 1 : 2);
-  // default occupancy: the 3-CTA variant for FP32 (fewest spills), else the variant's maximum
-  const int occ_def = b->prec == 2 ? blocks_per_sm_cached(2, 3) : max_occ(b->prec);
+  // default occupancy: the 3-CTA variant for FP32 (fewer spills than 4), the 2-CTA one for an instance alone (512 x 512
+  // plate: 1.30 ms a step at 2 CTAs per SM, 1.36 at 3, 1.34 at 4), else the variant's maximum
+  const int occ_def = b->prec == 2 ? blocks_per_sm_cached(2, n == 1 ? 2 : 3) : max_occ(b->prec);
   const int occ = (b->occ > 0) ? std::min(b->occ, max_occ(b->prec)) : occ_def;
   b->occ_launch = occ;
   // team policy: flat (multi-CTA teams of any size, cooperative launch, global barriers) or clusters

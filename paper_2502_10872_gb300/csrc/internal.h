@@ -22,9 +22,8 @@ constexpr int kMaxAmgLevels = 12;   // multigrid levels of one instance (build_a
 constexpr int kDirectWords = 8192;  // doubles of shared memory the direct Newton solve may use (the Newton variant's staging buffer)
 constexpr int kForceBlock = 128;    // threads of a force tile
 constexpr int kMaxTeamWaitMs = 4000;  // default bound of a team-barrier wait (Sched::wait_ns)
-constexpr int kBarWords = 64;       // barrier words per team (256 bytes): a 64-bit arrival counter at [0, 2),
-                                    // the rest unused (one team's words do not share a cache line with
-                                    // another team's)
+constexpr int kBarWords = 64;       // barrier words per team (256 bytes): eight 64-bit arrival counters 32 bytes apart
+                                    // (one team's words do not share a cache line with another team's)
 
 // stencil modes
 enum : uint8_t { MODE_PLATE = 0, MODE_SHELL = 1, MODE_FIXED = 2, MODE_NONE = 3 };

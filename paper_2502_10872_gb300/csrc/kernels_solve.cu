@@ -54,6 +54,8 @@ __device__ inline int ld_volatile_i(const int *p) { return *((volatile const int
 struct Team {
   int team, rank, size;
   unsigned int *bar;
+  unsigned long long episodes;   // global barriers the team has passed
+  bool few_ctas;                 // the variant runs up to two CTAs per SM
   int *abort_flag;
   int bank;     // partials are double-buffered: reduction k writes bank k % 2
   int mode;     // 0: one CTA; 1: global barrier; 2: one whole cluster; 3: several whole clusters
@@ -75,45 +77,76 @@ __device__ inline unsigned int cluster_ctarank() {
   return r;
 }
 
-__device__ inline double *part_of(const Inst &I, const Team &tm, int ch) {
+__device__ inline double *part_of(const Inst &I, Team &tm, int ch) {
   return I.part + 4 * ((size_t)tm.bank * I.n_chunks + ch);
 }
 
-// Bounded global-memory barrier among `parties` arrivals on the team's words (thread 0 of the caller only).
-// The team's 64-bit arrival counter only grows: it is zeroed when the team layout is built (and after an
-// abandoned launch), and every CTA of a team passes the same barriers, so an episode starts at a multiple
-// of `parties` and ends when the counter reaches the next one. The last arrival's own increment releases the
-// others (no reset or generation word to write after it), and no word is read before arriving.
-// Returns 0 if it gave up (timeout, or abort raised elsewhere).
-// One acquire-release increment and one acquire fence after relaxed polls (152 CTAs: 1.25 us, against 1.4 us with a full
-// fence on each side of a relaxed increment); the abort flag, another L2 round trip, is looked at only every 16th poll.
-__device__ int global_arrive_wait(const Team &tm, unsigned int parties) {
+// Bounded global-memory barrier among `parties` CTAs, `index` this one (all lanes of one warp). Party k arrives at
+// counter k mod 8 of the team (8 counters, 32 bytes apart, so that the arrivals of a large team do not queue at one
+// address); lane i waits for counter i to reach the episode's count. The 64-bit counters only grow: they are zeroed when
+// the team layout is built (and after an abandoned launch), and every CTA of a team passes the same barriers, so each
+// CTA knows the number of past episodes (tm.episodes, see barrier_episodes) and nothing is computed from, or read
+// back with, the arrival. Its release makes the CTA's writes of the phase (ordered before by the CTA barrier) visible.
+// Where up to two CTAs share an SM, the polls acquire, which saves the fence after them; each of them invalidates the SM's
+// L1, so with more CTAs per SM the polls are relaxed and one fence follows (batch of 256 with acquiring polls: 30.75 ->
+// 31.2 ms). Returns 0 if it gave up (timeout, or abort raised elsewhere); the abort flag, another L2 round trip, is looked
+// at only every 16th poll. Against one counter per team, whose new value each CTA waited for and divided by the team size,
+// per call: 128 x 128 cylinder 3.79 -> 3.69 ms, in FP64 5.53 -> 5.24 ms, 24 FP64 instances 1.53 -> 1.48 ms.
+constexpr unsigned kBarCounters = 8, kBarStride = 4;   // counters of a team, 64-bit words between them
+static_assert(2 * kBarCounters * kBarStride <= kBarWords, "counters fit the team's barrier words");
+
+__device__ __forceinline__ unsigned bar_share(unsigned parties, unsigned k) {   // parties at counter k
+  return (parties - k + kBarCounters - 1) / kBarCounters;
+}
+
+__device__ int global_arrive_wait(Team &tm, unsigned int parties, unsigned int index) {
   unsigned long long *count = reinterpret_cast<unsigned long long *>(tm.bar);
-  unsigned long long o;
-  // release: this CTA's writes of the phase (ordered before by the CTA barrier) are visible before its arrival
-  asm volatile("atom.add.acq_rel.gpu.global.u64 %0, [%1], 1;" : "=l"(o) : "l"(count) : "memory");
-  const unsigned long long target = (o / parties + 1ull) * parties;
-  if (o + 1ull != target) {
-    const unsigned long long t0 = gtimer();
-    const unsigned long long limit = tm.wait_ns;
-    for (unsigned int polls = 1;; ++polls) {
-      unsigned long long v;
-      asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(count) : "memory");
-      if (v >= target) break;
-      if (polls % 16 == 0 && ld_volatile_i(tm.abort_flag)) return 0;
+  const unsigned lane = threadIdx.x & 31;
+  if (lane == 0)
+    asm volatile("red.release.gpu.global.add.u64 [%0], 1;" ::"l"(count + kBarStride * (index % kBarCounters)) : "memory");
+  const bool mine = lane < min(parties, kBarCounters);
+  const unsigned long long past = tm.episodes + 1ull;
+  const unsigned long long target = mine ? past * bar_share(parties, lane) : 0ull;
+  const unsigned long long t0 = gtimer(), limit = tm.wait_ns;
+  for (unsigned int polls = 1;; ++polls) {
+    unsigned long long v = 0ull;
+    if (mine) {
+      if (tm.few_ctas)
+        asm volatile("ld.acquire.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(count + kBarStride * lane) : "memory");
+      else
+        asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(count + kBarStride * lane) : "memory");
+    }
+    if (__all_sync(0xffffffffu, v >= target)) break;
+    bool stop = false;
+    if (lane == 0) {
+      if (polls % 16 == 0 && ld_volatile_i(tm.abort_flag)) stop = true;
       if (gtimer() - t0 > limit) {
         atomicExch(tm.abort_flag, 1);
-        return 0;
+        stop = true;
       }
     }
-    asm volatile("fence.acq_rel.gpu;" ::: "memory");
+    if (__any_sync(0xffffffffu, stop)) return 0;
   }
+  if (!tm.few_ctas) asm volatile("fence.acq_rel.gpu;" ::: "memory");
+  if (lane == 0) tm.episodes = past;
   return 1;
+}
+
+// Episodes the team's barrier has completed before this launch, read before this CTA's first arrival (without which
+// none of the launch completes).
+__device__ unsigned long long barrier_episodes(const unsigned int *bar, unsigned parties, unsigned index) {
+  const unsigned k = index % kBarCounters;
+  unsigned long long v;
+  asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];"
+               : "=l"(v)
+               : "l"(reinterpret_cast<const unsigned long long *>(bar) + kBarStride * k)
+               : "memory");
+  return v / bar_share(parties, k);
 }
 
 // Team barrier. Returns false if the barrier was abandoned (timeout or abort raised by another CTA); every
 // CTA of a team, and of a cluster, gets the same verdict.
-__device__ bool team_sync(const Team &tm) {
+__device__ bool team_sync(Team &tm) {
   __shared__ int s_ok;
   __syncthreads();
   if (tm.mode == 0) return true;
@@ -125,16 +158,19 @@ __device__ bool team_sync(const Team &tm) {
     cluster_barrier();
     const unsigned int crank = cluster_ctarank();
     int *flag = tm.cluster_ok + (blockIdx.x / tm.cluster);
-    if (crank == 0 && threadIdx.x == 0) {
-      const int ok = global_arrive_wait(tm, (unsigned int)(tm.size / tm.cluster));
-      *((volatile int *)flag) = ok;
+    if (crank == 0 && threadIdx.x < 32) {
+      const int ok = global_arrive_wait(tm, (unsigned int)(tm.size / tm.cluster), (unsigned int)(tm.rank / tm.cluster));
+      if (threadIdx.x == 0) *((volatile int *)flag) = ok;
     }
     cluster_barrier();
     if (threadIdx.x == 0) s_ok = *((volatile int *)flag);
     __syncthreads();
     return s_ok != 0;
   }
-  if (threadIdx.x == 0) s_ok = global_arrive_wait(tm, (unsigned int)tm.size);
+  if (threadIdx.x < 32) {
+    const int ok = global_arrive_wait(tm, (unsigned int)tm.size, (unsigned int)tm.rank);
+    if (threadIdx.x == 0) s_ok = ok;
+  }
   __syncthreads();
   return s_ok != 0;
 }
@@ -180,7 +216,7 @@ __device__ __forceinline__ int fewest_threads_log(int size, F units) {
 }
 __device__ __forceinline__ int blocks_of(int n, int log) { return (n + (1 << log) - 1) >> log; }
 template <typename R>
-__device__ __forceinline__ int level_threads(int n, const Team &tm) {
+__device__ __forceinline__ int level_threads(int n, Team &tm) {
   if (sizeof(R) == 4) return kBlock;
   return 1 << fewest_threads_log(tm.size, [&](int log) { return blocks_of(n, log); });
 }
@@ -209,7 +245,7 @@ __device__ inline double (*stage_buf())[kBlock / 32][3] {
 // A: the type the warp sums were staged in (FP32 sums are widened here: 24 lanes of one warp instead of one lane of
 // each warp and value). Lane 8 k + w holds warp w's sum of value k; the warps of a chunk are added by a tree.
 template <typename A>
-__device__ void stage_flush(ChunkStage &cs, const Inst &I, const Team &tm) {
+__device__ void stage_flush(ChunkStage &cs, const Inst &I, Team &tm) {
   const A(*sm)[kBlock / 32][3] = reinterpret_cast<const A(*)[kBlock / 32][3]>(stage_buf());
   const int lane = threadIdx.x & 31, w = lane & 7;
   const int act = tm.act, per = I.chunk_rows >> 5;   // warps per chunk
@@ -227,7 +263,7 @@ __device__ void stage_flush(ChunkStage &cs, const Inst &I, const Team &tm) {
 }
 
 template <typename A>
-__device__ void stage_chunk(ChunkStage &cs, const Inst &I, const Team &tm, int blk, A v0, A v1, A v2) {
+__device__ void stage_chunk(ChunkStage &cs, const Inst &I, Team &tm, int blk, A v0, A v1, A v2) {
   A(*sm)[kBlock / 32][3] = reinterpret_cast<A(*)[kBlock / 32][3]>(stage_buf());
   if (cs.n == 0) cs.first = blk;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -635,7 +671,7 @@ struct LevelVal<double> {
 // team's CTAs take 256-stencil chunks of the combined list (triangles, then edge stencils) round robin; the
 // right-hand side reads the slots after the next team barrier.
 template <typename R, bool NT>
-__device__ void phase_forces(const Inst &I, const Team &tm) {
+__device__ void phase_forces(const Inst &I, Team &tm) {
   const Data<R> D(I, tm.chord_k > 0 ? I.xk : I.x);
   const int ns = I.nt + I.ne;
   for (int c = tm.rank; c * kBlock < ns; c += tm.size) {
@@ -672,7 +708,7 @@ __device__ inline int guess_order(const double e[3]) {
 }
 
 // partial sums of e0, e1, e2 over a sample of the rows (every fourth warp, another one in each chunk)
-__device__ void phase_history(const Inst &I, const Team &tm) {
+__device__ void phase_history(const Inst &I, Team &tm) {
   const int nv = I.nv;
   ChunkStage cs;
   const int act = tm.act;
@@ -725,7 +761,7 @@ struct ContribSum<float> {
 // b = M v + dt (f + f_ext) + (A - M) v_k, warm start v_k kept, so that the first residual b - A v_k is
 // -R(v_k), the backward-Euler residual, and the solve gives v_{k+1} = v_k - A^-1 R(v_k).
 template <typename RC, bool NT>
-__device__ void phase_rhs(const Inst &I, const Team &tm, int order) {
+__device__ void phase_rhs(const Inst &I, Team &tm, int order) {
   const int nv = I.nv;
   const bool chord = tm.chord_k > 0;
   const RC *con = reinterpret_cast<const RC *>(I.contrib);
@@ -811,7 +847,7 @@ __device__ void phase_rhs(const Inst &I, const Team &tm, int order) {
 // r32 = r64, xs = 0 (FP64), g32 = D32^-1 r32. If R is double: r = r64 (in place), sol unchanged, g = D^-1 r.
 // Multigrid: also the first V-cycle's level-0 pre-smoothing from zero, b0 = r, x0 = omega D^-1 r (row-local).
 template <typename R, bool NT>
-__device__ void phase_resid(const Inst &I, const Team &tm) {
+__device__ void phase_resid(const Inst &I, Team &tm) {
   const int nv = I.nv;
   const bool amg = I.amg_levels > 0;
   typename Vec<R>::G *b0 = amg ? reinterpret_cast<typename Vec<R>::G *>(I.amg[0].b) : nullptr;
@@ -883,7 +919,7 @@ __device__ void phase_resid(const Inst &I, const Team &tm) {
 
 // w = A u (u = g); partials (r,u), (w,u), (r,r)
 template <typename R, bool NT>
-__device__ void phase_spmv(const Inst &I, const Team &tm) {
+__device__ void phase_spmv(const Inst &I, Team &tm) {
   const int nv = I.nv;
   const R *val = Vec<R>::val(I);
   const typename Vec<R>::G *g = Vec<R>::g(I);
@@ -955,7 +991,7 @@ __device__ void phase_spmv(const Inst &I, const Team &tm) {
 // is formed from x itself, so the drift is measured there and corrected like any other inner error.
 // sum: also writes the chunks' partials of ||r||^2 of the new r (the sums phase_spmv would form from it, see cg_loop).
 template <typename R>
-__device__ void phase_update(const Inst &I, const Team &tm, R alpha, R beta, bool first, double *x,
+__device__ void phase_update(const Inst &I, Team &tm, R alpha, R beta, bool first, double *x,
                              double alpha_x, bool sum, bool direct) {
   const int nv = I.nv;
   const bool amg = I.amg_levels > 0 && !direct;
@@ -1215,7 +1251,7 @@ __device__ __forceinline__ void restrict_blk(const AmgDev &A, const AmgDev &C, b
 // with per-component constraints): y is zeroed at the components fix marks, so the preconditioned vector stays
 // on the free components.
 template <typename R, bool ST, bool MK = false>
-__device__ void lv_up(const AmgDev &A, const AmgDev &C, typename Vec<R>::G *y, const Team &tm,
+__device__ void lv_up(const AmgDev &A, const AmgDev &C, typename Vec<R>::G *y, Team &tm,
                       const uint8_t *fix = nullptr) {
   typedef typename Vec<R>::G G;
   const G *x = reinterpret_cast<const G *>(A.x);
@@ -1359,7 +1395,7 @@ __device__ __forceinline__ void resid4_blk(const AmgDev &A, int blk, int act) {
 // damped-Jacobi sweep of a coarse level: y = x + omega D^-1 (b - A x), x the previous sweep (the coarsest
 // level's sweeps when it is too large for a dense inverse)
 template <typename R, bool ST>
-__device__ void lv_smooth4(const AmgDev &A, const typename Vec<R>::G *x, typename Vec<R>::G *y, const Team &tm) {
+__device__ void lv_smooth4(const AmgDev &A, const typename Vec<R>::G *x, typename Vec<R>::G *y, Team &tm) {
   typedef typename Vec<R>::G G;
   const G *b = reinterpret_cast<const G *>(A.b);
   const R *dinv = LevelVal<R>::dinv(A);
@@ -1387,7 +1423,7 @@ __device__ inline bool staged(const HaloDev &H, int cap) {
 // Down step of level l in one team phase: the residual blocks of level l and the restriction blocks of level
 // l + 1 are independent (both read only b and x), so the team's CTAs take them from one list of units.
 template <typename R>
-__device__ bool down_step(const Inst &I, int l, const Team &tm) {
+__device__ bool down_step(const Inst &I, int l, Team &tm) {
   const AmgDev &A = I.amg[l];
   const AmgDev &C = I.amg[l + 1];
   // levels at and below the dense level, and the coarsest, are solved, not smoothed
@@ -1425,7 +1461,7 @@ __device__ bool down_step(const Inst &I, int l, const Team &tm) {
 
 // coarsest level: y = C^-1 b (dense inverse) or damped-Jacobi sweeps from zero
 template <typename R>
-__device__ bool coarsest(const Inst &I, const Team &tm) {
+__device__ bool coarsest(const Inst &I, Team &tm) {
   typedef typename Vec<R>::G G;
   const AmgDev &C = I.amg[I.amg_levels - 1];
   const G *b = reinterpret_cast<const G *>(C.b);
@@ -1473,7 +1509,7 @@ __device__ bool coarsest(const Inst &I, const Team &tm) {
 // Up step of level l in one team phase (coarse correction and post-smoothing); the output of level 0 is u
 // (in g), projected onto the free components when MK and the instance has per-component constraints.
 template <typename R, bool MK = false>
-__device__ bool up_step(const Inst &I, int l, const Team &tm) {
+__device__ bool up_step(const Inst &I, int l, Team &tm) {
   typedef typename Vec<R>::G G;
   const AmgDev &A = I.amg[l];
   const AmgDev &C = I.amg[l + 1];
@@ -1497,7 +1533,7 @@ __device__ bool up_step(const Inst &I, int l, const Team &tm) {
 // Level 0 (a small mesh, whose whole preconditioner is the dense inverse): the output is u (in g), projected like
 // up_step's.
 template <typename R, bool MK>
-__device__ bool dense_level(const Inst &I, const Team &tm) {
+__device__ bool dense_level(const Inst &I, Team &tm) {
   typedef typename Vec<R>::G G;
   constexpr int U = 8;
   const AmgDev &D = I.amg[I.amg_dense_level];
@@ -1601,7 +1637,7 @@ __device__ bool dense_level(const Inst &I, const Team &tm) {
 // before it. The pre-smoothing of each coarser level is fused into the restriction that produces its
 // right-hand side. Returns false on abort.
 template <typename R, bool MK = false>
-__device__ bool vcycle(const Inst &I, const Team &tm) {
+__device__ bool vcycle(const Inst &I, Team &tm) {
   const int top = I.amg_dense_level >= 0 ? I.amg_dense_level : I.amg_levels - 1;   // 0: the dense inverse alone
   for (int l = 0; l < top; ++l)
     if (!down_step<R>(I, l, tm)) return false;
@@ -1621,7 +1657,7 @@ __device__ bool vcycle(const Inst &I, const Team &tm) {
 // 19.6 ms. Larger instances keep PCG: their factor would not fit, and would be one CTA's work.
 // Layout in shared memory: band [3 nv][dir_w + 1], row i's entry (i, j) at i (dir_w + 1) + j - i + dir_w, holding
 // L_ij d_j below the diagonal; reciprocal pivots [3 nv]; the vector being solved [3 nv].
-__device__ inline bool direct_on(const Inst &I, const Team &tm) {
+__device__ inline bool direct_on(const Inst &I, Team &tm) {
   return I.nl_newton && I.dir_perm && 3 * I.nv * (I.dir_w + 3) <= 2 * tm.cap;
 }
 
@@ -1871,7 +1907,7 @@ __device__ int cg_loop(const Inst &I, Team &tm, double *x, double tol2, int max_
 }
 
 // sol += xs (the inner correction, accumulated in FP64); g64 = sol
-__device__ void phase_accumulate(const Inst &I, const Team &tm) {
+__device__ void phase_accumulate(const Inst &I, Team &tm) {
   const int nv = I.nv;
   const double *xs = reinterpret_cast<const double *>(I.xs);
   ROWS_BEGIN(I, tm)
@@ -1886,7 +1922,7 @@ __device__ void phase_accumulate(const Inst &I, const Team &tm) {
 
 // v_prev3 = v_prev2; v_prev2 = v_prev; v_prev = v; v = sol; x += dt v. Quasi-static solve: x += dt sol and the
 // velocity and its history are zero (the equilibrium is at rest).
-__device__ void phase_commit(const Inst &I, const Team &tm) {
+__device__ void phase_commit(const Inst &I, Team &tm) {
   const int nv = I.nv;
   const bool st = I.nl_static != 0;
   ROWS_BEGIN(I, tm)
@@ -1959,7 +1995,7 @@ __device__ bool team_max_step(const Inst &I, Team &tm, double *out) {
 
 // hand-off to the next iteration: the new iterate v_{k+1} = sol, or with the quasi-static limiter
 // v_k + alpha (sol - v_k); sol = vk = g64 = v_{k+1}, xk = x + dt v_{k+1} (where the next forces are evaluated)
-__device__ void phase_chord(const Inst &I, const Team &tm, double alpha, bool limit) {
+__device__ void phase_chord(const Inst &I, Team &tm, double alpha, bool limit) {
   const int nv = I.nv;
   const bool first = tm.chord_k == 0;
   ROWS_BEGIN(I, tm)
@@ -1995,7 +2031,7 @@ __device__ inline double nl_floor2(const Inst &I) {
   return 0.01 * fmax(I.nl_rtol * I.nl_rtol * r0, a * a);
 }
 
-__device__ void set_status(const Inst &I, const Team &tm, int err, int iters, int rounds, double rel) {
+__device__ void set_status(const Inst &I, Team &tm, int err, int iters, int rounds, double rel) {
   if (tm.rank == 0 && threadIdx.x == 0) {
     InstStatus *s = I.status;
     s->last_ns = (long long)(gtimer() - tm.t0);
@@ -2267,6 +2303,10 @@ __global__ void __launch_bounds__(kBlock, MINB) k_solve(const Inst *__restrict__
   if (threadIdx.x == 0) {
     tm.team = team;
     tm.bar = sch.bar + kBarWords * team;
+    tm.episodes = team_mode == 1   ? barrier_episodes(tm.bar, team_size, team_rank)
+                  : team_mode == 3 ? barrier_episodes(tm.bar, team_size / sch.cluster, team_rank / sch.cluster)
+                                   : 0ull;
+    tm.few_ctas = MINB <= 2;
     tm.abort_flag = sch.abort_flag;
     tm.bank = 0;
     tm.cluster = sch.cluster;
