@@ -507,16 +507,17 @@ bool band_inverse(const HostCsr &A, const std::vector<int32_t> &perm, int band, 
   return std::isfinite(cnorm) && eps * cnorm * snorm <= 0.25;
 }
 
-HostSell to_sell4(const HostCsr &M) {
+HostSell to_sell_lanes(const HostCsr &M, int lanes) {
+  const int m = 32 / lanes;   // rows of a slice
   HostSell S;
   S.n = M.n;
-  S.n_slices = (M.n + 7) / 8;
+  S.n_slices = (M.n + m - 1) / m;
   S.sl_ptr.assign(S.n_slices + 1, 0);
   for (int s = 0; s < S.n_slices; ++s) {
     int w = 0;
-    for (int i = 0; i < 8; ++i) {
-      const int r = s * 8 + i;
-      if (r < M.n) w = std::max(w, (M.ptr[r + 1] - M.ptr[r] + 3) / 4);
+    for (int i = 0; i < m; ++i) {
+      const int r = s * m + i;
+      if (r < M.n) w = std::max(w, (M.ptr[r + 1] - M.ptr[r] + lanes - 1) / lanes);
     }
     S.sl_ptr[s + 1] = S.sl_ptr[s] + 32 * w;
   }
@@ -524,9 +525,9 @@ HostSell to_sell4(const HostCsr &M) {
   S.sl_col.assign(nnz, 0);
   S.val.assign(nnz, 0.0);
   for (int r = 0; r < M.n; ++r) {
-    const int s = r / 8, i = r % 8;
+    const int s = r / m, i = r % m;
     for (int k = 0; k < M.ptr[r + 1] - M.ptr[r]; ++k) {
-      const int pos = S.sl_ptr[s] + 32 * (k / 4) + 4 * i + k % 4;
+      const int pos = S.sl_ptr[s] + 32 * (k / lanes) + lanes * i + k % lanes;
       S.sl_col[pos] = M.col[M.ptr[r] + k];
       S.val[pos] = M.val[M.ptr[r] + k];
     }

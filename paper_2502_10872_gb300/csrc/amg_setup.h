@@ -57,8 +57,14 @@ bool band_inverse(const HostCsr &A, const std::vector<int32_t> &perm, int band, 
 
 HostSell to_sell(const HostCsr &M);
 
-// SELL with 4 lanes per row (for the long rows of the restriction): slices of 8 rows; entry k of the slice's
-// row i (i = 0..7) sits at sl_ptr[s] + 32 (k / 4) + 4 i + k % 4, padding column 0 with value 0.
-HostSell to_sell4(const HostCsr &M);
+// SELL with `lanes` (4 or 16) lanes per row, for long rows: slices of m = 32 / lanes rows; entry k of the slice's row i
+// (i < m) sits at sl_ptr[s] + 32 (k / lanes) + lanes i + k % lanes, padding column 0 with value 0.
+HostSell to_sell_lanes(const HostCsr &M, int lanes);
+
+// Lanes per row of a restriction: 16 where its rows average 100 entries and more (the coarse levels: 130 to 190, against
+// 70 to 90 on level 0), which 4 lanes would load in five to seven dependent rounds. Per call, 4 -> 16 lanes (8 in
+// brackets): 128 x 128 cylinder 3.61 -> 3.41 ms (3.54 of 3.65), in FP64 5.16 -> 4.66 ms (4.96 of 5.26), 512 x 512 plate 13.9 ->
+// 13.2 ms, 12 serving requests 11.8 -> 11.5 ms; a batch of 256 on teams of 1 to 8 CTAs pays 1 % for the more blocks.
+inline int restriction_lanes(const HostCsr &Rs) { return Rs.n > 0 && Rs.val.size() >= 100 * (size_t)Rs.n ? 16 : 4; }
 
 }  // namespace shl

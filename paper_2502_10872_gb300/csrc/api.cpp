@@ -1003,17 +1003,18 @@ int setup_amg(shell_handle *h, const HostTopo &T, int mode, bool stage, const st
   }
   h->vcycle_bytes += 136 * (int64_t)H.levels[top].A.n;
   h->vcycle_bytes += 4 * (int64_t)(H.dense_level > 0 ? H.dense.size() : H.coarse_inv.size());
-  for (int l = 0; l < top; ++l) {   // down step: residual blocks and restriction blocks of 64 rows (level 0: 256)
-    const int n = H.levels[l].A.n, nn = H.levels[l + 1].A.n, per = kBlock / 4;
-    h->units = std::max(h->units, (l == 0 ? (n + kBlock - 1) / kBlock : (n + per - 1) / per) + (nn + per - 1) / per);
+  for (int l = 0; l < top; ++l) {   // down step: residual blocks (level 0: a thread per row) and restriction blocks
+    const int n = H.levels[l].A.n, nn = H.levels[l + 1].A.n;
+    const int ra = l == 0 ? kBlock : kBlock / 4, rr = kBlock / restriction_lanes(H.levels[l].Rs);
+    h->units = std::max(h->units, (n + ra - 1) / ra + (nn + rr - 1) / rr);
   }
   if (H.dense_level > 0) h->units = std::max(h->units, (H.dense_n + 7) / 8);
   std::vector<HostSell> As(L), Ps(L), Rs(L);
   for (int l = 0; l < L; ++l) {
-    if (l > 0) As[l] = to_sell4(H.levels[l].A);
+    if (l > 0) As[l] = to_sell_lanes(H.levels[l].A, 4);
     if (l < L - 1) {
       Ps[l] = to_sell(H.levels[l].Ps);
-      Rs[l] = to_sell4(H.levels[l].Rs);
+      Rs[l] = to_sell_lanes(H.levels[l].Rs, restriction_lanes(H.levels[l].Rs));
     }
   }
   // gather lists for the FP32 products (level 0 shares the instance's)
@@ -1024,7 +1025,7 @@ int setup_amg(shell_handle *h, const HostTopo &T, int mode, bool stage, const st
     if (l > 0) build_halo(V.A.n, V.A.n, As[l].sl_ptr, As[l].sl_col, V.A.ptr, true, &Ha[l], 4);
     if (l < L - 1) {
       build_halo(V.Ps.n, V.Ps.m, Ps[l].sl_ptr, Ps[l].sl_col, V.Ps.ptr, false, &Hp[l]);
-      build_halo(V.Rs.n, V.Rs.m, Rs[l].sl_ptr, Rs[l].sl_col, V.Rs.ptr, false, &Hr[l], 4);
+      build_halo(V.Rs.n, V.Rs.m, Rs[l].sl_ptr, Rs[l].sl_col, V.Rs.ptr, false, &Hr[l], restriction_lanes(V.Rs));
     }
   }
   const int nc = H.levels[L - 1].A.n;
@@ -1040,6 +1041,7 @@ int setup_amg(shell_handle *h, const HostTopo &T, int mode, bool stage, const st
       D.n_next = (l < L - 1) ? H.levels[l + 1].A.n : 0;
       D.omega = H.levels[l].omega;
       D.omega32 = float(D.omega);
+      D.r_log = l < L - 1 && restriction_lanes(H.levels[l].Rs) == 16 ? 4 : 2;
       if (l > 0) {
         D.a_ptr = C.take<int32_t>(As[l].sl_ptr.size());
         D.a_col = C.take<int32_t>(As[l].sl_col.size());

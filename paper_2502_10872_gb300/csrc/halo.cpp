@@ -8,7 +8,7 @@ namespace shl {
 bool build_halo(int n_rows, int n_cols, const std::vector<int32_t> &sl_ptr, const std::vector<int32_t> &sl_col,
                 const std::vector<int32_t> &row_ptr, bool square, HostHalo *out, int lanes) {
   *out = HostHalo();
-  if (n_rows <= 0 || n_cols <= 0 || (lanes != 1 && lanes != 4)) return false;
+  if (n_rows <= 0 || n_cols <= 0 || (lanes != 1 && lanes != 4 && lanes != 16)) return false;
   const int rows_blk = kHaloBlock / lanes, rows_slice = 32 / lanes;
   // position of entry k of row r in the SELL layout
   auto pos_of = [&](int r, int k) {

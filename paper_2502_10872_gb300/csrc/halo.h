@@ -24,7 +24,7 @@ struct HostHalo {
 
 // row_ptr: CSR row offsets of the matrix (row r has row_ptr[r+1] - row_ptr[r] stored entries, the first ones
 // of its SELL row). lanes: lanes per row of the SELL layout (1: SELL-32, slices of 32 rows, 256-row blocks;
-// 4: slices of 8 rows with 4 lanes each, 64-row blocks). Returns false (out left empty) if a list would not
+// 4, 16: slices of 32 / lanes rows, blocks of 256 / lanes rows). Returns false (out left empty) if a list would not
 // fit 16-bit local indices.
 bool build_halo(int n_rows, int n_cols, const std::vector<int32_t> &sl_ptr, const std::vector<int32_t> &sl_col,
                 const std::vector<int32_t> &row_ptr, bool square, HostHalo *out, int lanes = 1);

@@ -60,7 +60,7 @@ struct HaloDev {
 
 // One level of the smoothed-aggregation multigrid preconditioner (device pointers). P (rows of this level ->
 // columns of the next) and the level-0 operator are SELL-32; R = P^T (rows of the next level -> columns of
-// this one) and the coarse operators A (levels >= 1), whose rows are long, are SELL with 4 lanes per row
+// this one; 4 or 16 lanes per row) and the coarse operators A (levels >= 1), whose rows are long, are SELL with 4 lanes per row
 // (slices of 8 rows, entry k of slice row i at ptr[s] + 32 (k / 4) + 4 i + k % 4), with gather lists over
 // 64-row blocks. Level vectors are array-of-structures [n][4] in the solve precision.
 struct AmgDev {
@@ -74,11 +74,12 @@ struct AmgDev {
   int32_t *p_ptr, *p_col;        // Ps = (I - omega D^-1 A) P, SELL-32 (fine rows -> next level's columns)
   float *p_val32;
   double *p_val64;
-  int32_t *r_ptr, *r_col;        // Rs = R (I - omega A D^-1) = Ps^T, 4 lanes per row
+  int32_t *r_ptr, *r_col;        // Rs = R (I - omega A D^-1) = Ps^T, 2^r_log lanes per row
   float *r_val32;
   double *r_val64;
   double omega;                  // damped-Jacobi weight
-  float omega32, pad;            // the same, rounded
+  float omega32;                 // the same, rounded
+  int32_t r_log;                 // log2 of R's lanes per row (2 or 4)
   void *b, *x, *r, *y;           // right-hand side, pre-smoothed x, its residual, cycle output (AoS)
   HaloDev ha, hp, hr;            // gather lists of A, Ps and Rs (FP32 products)
 };

@@ -1171,9 +1171,10 @@ __device__ __forceinline__ void resid_blk(const AmgDev &A, int blk, int act) {
   rr[row] = Vec<R>::mk(R(bi.x) - ax, R(bi.y) - ay, R(bi.z) - az);
 }
 
-// restriction of one 64-row block of the next level with its pre-smoothing from zero fused: bc = Rs b;
-// xc = omega_c Dc^-1 bc. Rs has 4 lanes per row (its rows are long): lane k % 4 of a row sums the entries
-// k, k + 4, ... in increasing order, and the four partial sums are added in a fixed shuffle tree; staged
+// restriction of one block of the next level's rows with its pre-smoothing from zero fused: bc = Rs b;
+// xc = omega_c Dc^-1 bc. Rs has m = 4 or 16 lanes per row (its rows are long, see restriction_lanes), so a block has 64 or
+// 16 rows: lane k % m of a row sums the entries k, k + m, ... in increasing order, and the partial sums are added in a
+// fixed shuffle tree; staged
 // (FP32) and unstaged products run the same arithmetic. The loads that do not depend on the staged vector
 // (slice bounds, first nonzeros) are issued before the staging barrier.
 template <typename R, bool ST>
@@ -1189,11 +1190,12 @@ __device__ __forceinline__ void restrict_blk(const AmgDev &A, const AmgDev &C, b
   const R omc = LevelVal<R>::omega(C);
   const int n = A.n_next;
   const int lane = threadIdx.x & 31;
-  const int row = blk * (act / 4) + (int)(threadIdx.x >> 2);
+  const int rl = A.r_log;
+  const int row = blk * (act >> rl) + (int)(threadIdx.x >> rl);
   const bool valid = row < n;
   int p = 0, b1 = 0;
   if (valid) {
-    const int s = row >> 3;
+    const int s = row >> (5 - rl);
     p = A.r_ptr[s] + lane;
     b1 = A.r_ptr[s + 1];
   }
@@ -1238,7 +1240,15 @@ __device__ __forceinline__ void restrict_blk(const AmgDev &A, const AmgDev &C, b
   ax += __shfl_xor_sync(0xffffffffu, ax, 2);
   ay += __shfl_xor_sync(0xffffffffu, ay, 2);
   az += __shfl_xor_sync(0xffffffffu, az, 2);
-  if (valid && (threadIdx.x & 3) == 0) {
+  if (rl == 4) {
+    ax += __shfl_xor_sync(0xffffffffu, ax, 4);
+    ay += __shfl_xor_sync(0xffffffffu, ay, 4);
+    az += __shfl_xor_sync(0xffffffffu, az, 4);
+    ax += __shfl_xor_sync(0xffffffffu, ax, 8);
+    ay += __shfl_xor_sync(0xffffffffu, ay, 8);
+    az += __shfl_xor_sync(0xffffffffu, az, 8);
+  }
+  if (valid && (threadIdx.x & ((1 << rl) - 1)) == 0) {
     bc[row] = Vec<R>::mk(ax, ay, az);
     if (pre) {
       const R d = omc * dinvc[row];
@@ -1429,10 +1439,10 @@ __device__ bool down_step(const Inst &I, int l, Team &tm) {
   // levels at and below the dense level, and the coarsest, are solved, not smoothed
   const int top = I.amg_dense_level > 0 ? I.amg_dense_level : I.amg_levels - 1;
   const bool pre = l + 1 < top;
-  // residual blocks of act rows (4 threads a row on the coarse levels) and restriction blocks of act / 4 rows
-  const int n = A.n, nn = A.n_next;
+  // residual blocks of act rows (4 threads a row on the coarse levels) and restriction blocks
+  const int n = A.n, nn = A.n_next, rl = A.r_log;
   auto resids = [&](int log) { return blocks_of(n, l == 0 ? log : log - 2); };
-  auto units = [&](int log) { return resids(log) + blocks_of(nn, log - 2); };
+  auto units = [&](int log) { return resids(log) + blocks_of(nn, log - rl); };
   const int log = sizeof(R) == 4 ? kBlockLog : fewest_threads_log(tm.size, units);
   const int act = 1 << log, nf = resids(log), nu = units(log);
   const bool sa = staged<R>(A.ha, tm.cap), sr = staged<R>(A.hr, tm.cap);
