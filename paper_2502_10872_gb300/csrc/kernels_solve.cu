@@ -1,6 +1,7 @@
 // kernels_solve.cu -- persistent step kernel: per-stencil forces, right-hand side, preconditioned conjugate
 // gradients on the constant matrix (Jacobi, or a smoothed-aggregation multigrid V-cycle with its damped-Jacobi
-// sweeps folded into the transfers and one dense operator for its coarse end), state update. One launch per
+// sweeps folded into the transfers and one dense operator for its coarse end, or a small mesh's dense inverse), state
+// update. Small FP64 Newton systems are factored (direct_factor). One launch per
 // step serves every instance of a batch; each team evaluates its own FP32 instance's stencils before its solve
 // (FP64 instances take their forces from the standalone force launch just before).
 //
@@ -25,8 +26,8 @@
 // per level above its dense end and one for that end):
 //   p = u + beta p; s = w + beta s; x += alpha p; r -= alpha s; u = D^-1 r; w = A u;
 //   gamma' = (r,u); delta' = (w,u); beta' = gamma'/gamma; alpha' = gamma'/(delta' - beta' gamma'/alpha).
-// Warm start: the velocity extrapolated from the last ones (cubic while they are one motion, see guess_order). FP64 mode: one CG in FP64 from it, until
-// ||r|| <= rtol ||b||.
+// Warm start: the velocity extrapolated from the last ones (cubic while they are one motion, see guess_order).
+// FP64 mode: one CG in FP64 from it, until ||r|| <= rtol ||b||.
 // FP32 refinement mode: r64 = b - A v in FP64 (FP64 matrix and vector); inner CG in FP32 on A d = r64 from
 // d = 0 to a relative tolerance (or to a margin below the refinement target, if that is reached first);
 // v += d; repeat until ||r64|| <= refine_rtol ||b||.
@@ -227,7 +228,7 @@ __device__ inline int row_threads(const Inst &I, int size) {
   return max(I.chunk_rows, 1 << fewest_threads_log(size, [&](int log) { return blocks_of(nv, log); }));
 }
 
-// Per-chunk partials: each chunk's (chunk_rows rows') three values are reduced by a fixed tree (warp shuffles, then the
+// Per-chunk partials: each chunk's (chunk_rows rows) three values are reduced by a fixed tree (warp shuffles, then the
 // warps' sums). The warp sums of up to kStage passes are staged in shared memory and written out together, so
 // a CTA that makes several passes in a phase pays two __syncthreads per kStage passes instead of per pass.
 constexpr int kStage = 32;
