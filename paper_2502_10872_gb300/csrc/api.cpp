@@ -879,7 +879,7 @@ std::vector<double> to_soa(const double *aos, int nv) {
 // (and, like it, from 256 vertices on: below, callers that cap the iterations rely on Jacobi's). It replaces 7 to 15 iterations of six phases each by one or two of three, so it pays
 // until one CTA's read of the inverse (4 n^2 bytes from L2, 16 k clocks at n = 512) costs as much as those iterations;
 // the limit lies there because the set-up (7 ms of one host core at n = 529, 2 ms at 289) grows with n^2 times the
-// band. Per call: 289-vertex plate 343 -> 159 us, 450-vertex panel in FP64 740 -> 125 us, 24 FP64 instances of 81 to
+// band. Per call: 289-vertex plate 343 -> 159 us (149 now), 450-vertex panel in FP64 740 -> 125 us, 24 FP64 instances of 81 to
 // 4,225 vertices 3.05 -> 2.64 ms, batch of 256 31.4 -> 31.0 ms. Leaves amg_levels at 0 where the inverse cannot be held in the solve's precision (see band_inverse).
 constexpr int kDenseRows = 512;
 int setup_dense(shell_handle *h, const HostCsr &A, const HostTopo &T) {
