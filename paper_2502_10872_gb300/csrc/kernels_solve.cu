@@ -1885,6 +1885,9 @@ __device__ int cg_loop(const Inst &I, Team &tm, double *x, double tol2, int max_
       }
       if (!team_sync(tm)) return -2;
       direct = __ldcg(reinterpret_cast<const double *>(I.w)) != 0.0;
+      // every thread has read the verdict before the first product overwrites it: without the factor and with the
+      // Jacobi preconditioner no other barrier lies between
+      if (!team_sync(tm)) return -2;
     }
   }
   for (int it = 0;; ++it) {
