@@ -405,7 +405,9 @@ int rebuild_tables(shell_batch *b) {
     // row blocks take anyway reach (more would only lengthen the barriers). With the dense level's split among many
     // CTAs (dense_level), per call: 24 x 17 panel in FP64 958 -> 737 us, 97 x 62 Jacobi case 780 -> 678 us, 128 x 128
     // cylinder 4.33 -> 3.94 ms, in FP64 7.38 -> 6.15 ms, 512 x 512 plate 13.1 -> 12.2 ms. An instance of one row block
-    // keeps its one CTA, whose barriers cost nothing, unless it has a dense product to share out.
+    // keeps its one CTA, whose barriers cost nothing, unless it has a dense product to share out. The team does not
+    // depend on the measured time, so there is nothing to re-plan (plan_T is the time of the team planned above: kept, it
+    // had the tables of 1,024 row blocks, planned at 256 CTAs and run on 304, rebuilt on every call).
     if (n == 1) {
       const shell_handle *h = b->slots[b->active[0]];
       const int sms = num_sms(), blocks = cmax(0);
@@ -417,6 +419,7 @@ int rebuild_tables(shell_batch *b) {
       team_inst = {{0}};
       queue.clear();
       used = team_size[0];
+      b->plan_T = 0.0;
     }
   }
   if (CS) {
