@@ -548,10 +548,20 @@ int launch_step(shell_batch *b) {
   return SHELL_OK;
 }
 
+// Enqueues the read-back of the active instances' statuses and of the launches' abort flag, gathered by one kernel.
+int enqueue_statuses(shell_batch *b, InstStatus *out, int32_t *aborted) {
+  cudaStream_t st = b->mem.st;
+  CK(launch_gather_status(b->d_insts, b->n_active, b->d_status_out, b->sched.abort_flag, b->d_abort_out, st));
+  CK(cudaMemcpyAsync(out, b->d_status_out, sizeof(InstStatus) * b->n_active, cudaMemcpyDeviceToHost, st));
+  CK(cudaMemcpyAsync(aborted, b->d_abort_out, sizeof(int32_t), cudaMemcpyDeviceToHost, st));
+  return SHELL_OK;
+}
+
 // A step that may take many Newton or chord iterations (a quasi-static solve allows 1,000) is launched in groups, and
-// ends after the group in which its last instance stopped: the cantilever's 48 iterations took 1,001 pairs of
-// launches, recorded into a graph again on every call. A group costs one read of the statuses, about as much as two
-// launches of instances that are done, so it pays from a few times that many on.
+// ends after the group in which its last instance stopped, or a wait gave up (the launches after it could only wait
+// again): the cantilever's 48 iterations took 1,001 pairs of launches, recorded into a graph again on every call. A
+// group costs one read of the statuses, about as much as four launches of instances that are done, so it pays from a
+// few times that many on.
 constexpr int kChordGroup = 12;
 int launch_step_groups(shell_batch *b) {
   cudaStream_t st = b->mem.st;
@@ -563,16 +573,14 @@ int launch_step_groups(shell_batch *b) {
       CK(solve_launch(b, st, k));
     }
     if (k == b->chord_max) break;
-    bool more = false;
-    for (int q = 0; q < b->n_active; ++q) {
-      const Inst &I = b->slots[b->active[q]]->h;
-      now[q].err = SHELL_OK;
-      now[q].nl_flags = 0;
-      if (I.nl_max > k) CK(cudaMemcpyAsync(&now[q], I.status, sizeof(InstStatus), cudaMemcpyDeviceToHost, st));
-    }
+    int32_t aborted = 0;
+    const int rc = enqueue_statuses(b, now.data(), &aborted);
+    if (rc != SHELL_OK) return rc;
     CK(cudaStreamSynchronize(st));
-    for (const InstStatus &s : now) more = more || (s.err == SHELL_OK && (s.nl_flags & 1));
-    if (!more) break;
+    bool more = false;
+    for (int q = 0; q < b->n_active; ++q)
+      more = more || (b->slots[b->active[q]]->h.nl_max > k && now[q].err == SHELL_OK && (now[q].nl_flags & 1));
+    if (!more || aborted) break;
   }
   return SHELL_OK;
 }
@@ -724,10 +732,11 @@ int batch_step(shell_batch *b, int n_steps, shell_step_stats *stats, const doubl
     int rc = enqueue_states(b, xout, vout, nullptr, nullptr);
     if (rc != SHELL_OK) return rc;
   }
-  CK(launch_gather_status(b->d_insts, n, b->d_status_out, b->sched.abort_flag, b->d_abort_out, st));
   int32_t aborted = 0;
-  CK(cudaMemcpyAsync(after.data(), b->d_status_out, sizeof(InstStatus) * n, cudaMemcpyDeviceToHost, st));
-  CK(cudaMemcpyAsync(&aborted, b->d_abort_out, sizeof(int32_t), cudaMemcpyDeviceToHost, st));
+  {
+    int rc = enqueue_statuses(b, after.data(), &aborted);
+    if (rc != SHELL_OK) return rc;
+  }
   CK(cudaStreamSynchronize(st));
   b->kern_ms[0] = b->kern_ms[1] = 0.0;
   for (int s = 0; s < n_prof * b->chord_max; ++s) {

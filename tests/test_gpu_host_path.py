@@ -43,3 +43,45 @@ def test_a_large_instance_alone_is_planned_once():
     for _ in range(3):
         gb.shell_step(h, 1)
     assert activity(lambda: [gb.shell_step(h, 1) for _ in range(3)])["Memcpy HtoD"] == 0
+
+
+def chord(sc, iters):
+    h = gb.create_from_scenario(sc, precision="fp32_refine")
+    gb.shell_set_nonlinear(h, iters, 0.0)   # no tolerance: every iteration runs
+    return h
+
+
+def test_a_group_of_chord_iterations_reads_the_statuses_at_once():
+    """60 iterations are five groups: four reads between them and the call's own, two copies each, however many
+    instances the batch holds."""
+    b = gb.shell_batch_create(1 << 40)
+    hs = [chord(sg.plate_clamped_x0(9 + k, model="EP"), 60) for k in range(8)]
+    for h in hs:
+        gb.shell_batch_admit(b, h)
+    gb.shell_batch_step(b, 1)
+    counts = activity(lambda: gb.shell_batch_step(b, 1))
+    assert sum(n for k, n in counts.items() if "k_solve" in k) == 60
+    assert counts["Memcpy DtoH"] <= 10
+    gb.shell_batch_destroy(b)
+
+
+def test_a_wait_that_gave_up_ends_the_chord_iterations():
+    """A team whose barrier wait runs out (1 ns) launches no further group, commits nothing, and steps on after."""
+    sc = sg.cylinder_panel(48, "FS", ny=40)
+    ref, h = chord(sc, 60), chord(sc, 60)
+    b = gb.shell_batch_create(1 << 40)
+    slot = gb.shell_batch_admit(b, h)
+    gb.shell_batch_step(b, 1)
+    gb.shell_batch_set_wait_limit(b, 1)
+    out = []
+    counts = activity(lambda: out.append(gb.shell_batch_step(b, 1, check=False)))
+    rc, stats = out[0]
+    assert rc == gb.SHELL_ERR_TIMEOUT and stats[slot]["steps_done"] == 0
+    assert sum(n for k, n in counts.items() if "k_solve" in k) == 12
+    gb.shell_batch_set_wait_limit(b, 0)
+    rc, stats = gb.shell_batch_step(b, 1)
+    assert rc == 0 and stats[slot]["steps_done"] == 1
+    gb.shell_step(ref, 2)
+    for a, c in zip(gb.shell_get_state(ref), gb.shell_batch_get_states(b)):
+        assert (a == c).all()
+    gb.shell_batch_destroy(b)
