@@ -407,8 +407,10 @@ int rebuild_tables(shell_batch *b) {
     // cylinder 4.33 -> 3.94 ms, in FP64 7.38 -> 6.15 ms, 512 x 512 plate 13.1 -> 12.2 ms. An instance of one row block
     // keeps its one CTA, whose barriers cost nothing, unless it has a dense product to share out. The team does not
     // depend on the measured time, so there is nothing to re-plan (plan_T is the time of the team planned above: kept, it
-    // had the tables of 1,024 row blocks, planned at 256 CTAs and run on 304, rebuilt on every call).
-    if (n == 1) {
+    // had the tables of 1,024 row blocks, planned at 256 CTAs and run on 304, rebuilt on every call). The CTA share keeps
+    // its say where it has one: below beta = 1 the model gives an instance alone as many CTAs as it has blocks whatever the
+    // share, from there on (a share of 25 and more) one.
+    if (n == 1 && beta < 1.0) {
       const shell_handle *h = b->slots[b->active[0]];
       const int sms = num_sms(), blocks = cmax(0);
       const int per_sm = std::min(occ, (blocks + sms - 1) / sms);

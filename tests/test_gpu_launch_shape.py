@@ -1,0 +1,29 @@
+"""Launch shapes set by the caller or tried by the autotuner."""
+import pytest
+
+import shellgen as sg
+
+gb = pytest.importorskip("paper_2502_10872_gb300")
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _cuda():
+    import torch
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    gb.load_library()
+
+
+@pytest.mark.parametrize("precision", ["fp64", "fp32_refine"])
+def test_the_share_sets_the_team_of_an_instance_alone(precision):
+    """Shares at which a second CTA costs more than it saves in the planner's model (25 and more) give one CTA."""
+    for share, one in ((1.0, False), (20.0, False), (30.0, True)):
+        h = gb.create_from_scenario(sg.cylinder_panel(48, "FS", ny=40), precision=precision)
+        b = gb.shell_batch_create(1 << 40)
+        slot = gb.shell_batch_admit(b, h)
+        gb.shell_batch_set_launch(b, 2, share)
+        for _ in range(2):
+            rc, stats = gb.shell_batch_step(b, 1)
+            assert rc == 0 and (stats[slot]["team_ctas"] == 1) == one, share
+        gb.shell_batch_destroy(b)
