@@ -351,8 +351,8 @@ int shell_batch_step_times(shell_batch *b, float *out_ms, int32_t n);
  * launch) and out_ms[1] = summed time of the step launches of the last call, in milliseconds. */
 int shell_batch_set_profiling(shell_batch *b, int32_t on);
 /* Autotune the persistent solve launch of this batch: flat teams (any size, global barriers, cooperative
- * launch) with 3 occupancies (CTAs per SM: 1, half, the maximum) x 3 CTA shares for large instances (x0.5,
- * x1, x2), and one-cluster teams (8-CTA thread-block clusters, hardware cluster barrier) with the 3 shares;
+ * launch) with up to 3 occupancies (CTAs per SM: 1, half, the maximum; 2, 3 and 4 in a batch of FP32-refinement
+ * instances without Newton iterations or per-component constraints) x 3 CTA shares for large instances (x0.5, x1, x2), and one-cluster teams (8-CTA thread-block clusters, hardware cluster barrier) with the 3 shares;
  * steps_per_trial real (committed) steps each; keeps the fastest by device time, then runs 3 more calls of
  * steps_per_trial steps with it, re-planning the teams from that shape's own measured times (so a call takes
  * (trials that ran + 3) x steps_per_trial committed steps). A batch's results do not

@@ -1917,10 +1917,8 @@ int shell_batch_autotune(shell_batch *b, int32_t steps_per_trial, double *out_ms
   if (b->n_active == 0) return SHELL_OK;
   const int occ_max = max_occ(b->prec);
   int occs[3] = {1, std::max(1, occ_max / 2), occ_max};
-  if (b->prec == 2) {   // the FP32 variants compiled for 3 and 4 CTAs per SM
-    occs[0] = blocks_per_sm_cached(2, 3);
-    occs[1] = occs[2] = blocks_per_sm_cached(2, 4);
-  }
+  if (b->prec == 2)   // the FP32 variants compiled for 2, 3 and 4 CTAs per SM
+    for (int k = 0; k < 3; ++k) occs[k] = blocks_per_sm_cached(2, 2 + k);
   const double scales[3] = {0.5, 1.0, 2.0};
   double best = 1e300;
   int best_k = 0;

@@ -27,3 +27,14 @@ def test_the_share_sets_the_team_of_an_instance_alone(precision):
             rc, stats = gb.shell_batch_step(b, 1)
             assert rc == 0 and (stats[slot]["team_ctas"] == 1) == one, share
         gb.shell_batch_destroy(b)
+
+
+def test_the_autotuner_tries_three_occupancies_in_fp32():
+    b = gb.shell_batch_create(1 << 40)
+    hs = [gb.create_from_scenario(sc, precision="fp32_refine") for sc in sg.mixed_batch(6, seed=3, side_lo=6, side_hi=40)]
+    for h in hs:
+        gb.shell_batch_admit(b, h)
+    info = gb.shell_batch_autotune(b, 1)
+    assert all(ms > 0.0 for ms in info["trial_ms"][:9])
+    assert info["ctas_per_sm"] in (2, 3, 4)
+    gb.shell_batch_destroy(b)
