@@ -879,22 +879,21 @@ std::vector<double> to_soa(const double *aos, int nv) {
   return s;
 }
 
-// Multigrid preconditioner: download the assembled FP64 matrix, build the smoothed-aggregation hierarchy
-// on the host (the matrix is constant, so this happens once) and upload its levels: the transfers with the
-// smoother folded in (Ps in SELL-32, Rs with 4 lanes per row), the coarse operators with 4 lanes per row,
-// the dense operator of the coarse end of the cycle, and (FP32 instances) the gather lists of every product.
-// Per-component constraints (fixb: fixed-component bits per vertex, empty if none has fixed and free ones): the
-// hierarchy is built from A with the diagonal of each such vertex doubled. A itself can be nearly singular then
-// (with nothing pinned, a rigid motion costs only its mass), and a cycle of A amplifies those motions, which the
-// projected system has removed; the doubled diagonal ties the constrained vertices down instead. Level 0 then
-// carries that matrix's values, and the instance's inverse diagonal (Jacobi, and the level-0 pre-smoothing
-// done in the residual and update phases) becomes its own, so the cycle stays symmetric.
-// Small meshes: the inverse of the step matrix as the preconditioner, one dense product in place of a multigrid cycle
-// (and, like it, from 256 vertices on: below, callers that cap the iterations rely on Jacobi's). It replaces 7 to 15 iterations of six phases each by one or two of three, so it pays
-// until one CTA's read of the inverse (4 n^2 bytes from L2, 16 k clocks at n = 512) costs as much as those iterations;
-// the limit lies there because the set-up (7 ms of one host core at n = 529, 2 ms at 289) grows with n^2 times the
-// band. Per call: 289-vertex plate 343 -> 159 us (149 now), 450-vertex panel in FP64 740 -> 125 us, 24 FP64 instances of 81 to
-// 4,225 vertices 3.05 -> 2.64 ms, batch of 256 31.4 -> 31.0 ms. Leaves amg_levels at 0 where the inverse cannot be held in the solve's precision (see band_inverse).
+// Small meshes: the inverse of the step matrix as the preconditioner, one dense product in place of a multigrid cycle. It
+// replaces 8 to 20 iterations of six phases each by one or two of three. Leaves amg_levels at 0 where the inverse cannot be
+// held in the solve's precision (see band_inverse). Per call: 289-vertex plate 343 -> 177 us, 450-vertex panel in FP64
+// 740 -> 125 us, 24 FP64 instances of 81 to 4,225 vertices 3.05 -> 2.64 ms, batch of 256 31.4 -> 31.0 ms.
+// Limits, both sides measured: 4 steps from a given state, stiff plate in FP32 and panel in FP64, cycle -> inverse.
+//   vertices                      552            784            961            1,122
+//   alone, FP32, us           1219 -> 462    1196 -> 474    1200 -> 474    1224 -> 483    (506 vertices: 464)
+//   alone, FP64, us           2628 -> 377    2655 -> 400    2661 -> 401    2708 -> 415                  (367)
+//   24 in a batch, FP32, us    526 -> 449     557 -> 605     573 -> 817     670 -> 903                  (485)
+//   24 in a batch, FP64, us   1892 -> 554    2312 -> 858   2443 -> 1072   2589 -> 1161                  (528)
+//   shell_create, ms           1.8 -> 2.8     2.7 -> 5.6     3.5 -> 8.6    4.3 -> 12.0                  (2.4)
+// A call alone would gain at every size measured, a batch in FP32 up to some 650 vertices; the upper limit is where the
+// set-up, which grows with n^2 times the band, costs no more than about one such call saves. The lower limit is the
+// cycle's own: below 256 vertices the automatic choice is Jacobi's iteration, which callers that cap the iterations rely
+// on (225 vertices, Jacobi -> inverse: 2004 -> 428 us in FP32, 3780 -> 363 us in FP64, shell_create 0.4 -> 0.8 ms).
 constexpr int kDenseRows = 512;
 int setup_dense(shell_handle *h, const HostCsr &A, const HostTopo &T) {
   Inst &I = h->h;
@@ -957,6 +956,16 @@ int setup_dense(shell_handle *h, const HostCsr &A, const HostTopo &T) {
   return SHELL_OK;
 }
 
+// Multigrid preconditioner: download the assembled FP64 matrix, build the smoothed-aggregation hierarchy
+// on the host (the matrix is constant, so this happens once) and upload its levels: the transfers with the
+// smoother folded in (Ps in SELL-32, Rs with 4 lanes per row), the coarse operators with 4 lanes per row,
+// the dense operator of the coarse end of the cycle, and (FP32 instances) the gather lists of every product.
+// Per-component constraints (fixb: fixed-component bits per vertex, empty if none has fixed and free ones): the
+// hierarchy is built from A with the diagonal of each such vertex doubled. A itself can be nearly singular then
+// (with nothing pinned, a rigid motion costs only its mass), and a cycle of A amplifies those motions, which the
+// projected system has removed; the doubled diagonal ties the constrained vertices down instead. Level 0 then
+// carries that matrix's values, and the instance's inverse diagonal (Jacobi, and the level-0 pre-smoothing
+// done in the residual and update phases) becomes its own, so the cycle stays symmetric.
 int setup_amg(shell_handle *h, const HostTopo &T, int mode, bool stage, const std::vector<uint8_t> &fixb) {
   Inst &I = h->h;
   cudaStream_t st = h->mem.st;
@@ -1276,7 +1285,8 @@ int shell_create(const shell_mesh *mesh, const shell_material *mat, int32_t mode
   I.precision = opt.precision;
   I.kt = T.kt;
   I.n_slices = T.n_slices;
-  // FP64 instances split into chunks of down to a warp's rows, at most about one per SM (see row_threads)
+  // FP64 instances split into chunks of down to a warp's rows, at most about one per SM (see row_threads). The number is a
+  // constant, not the device's: the chunks set the order of the sums, and with it the result's last bits.
   I.chunk_rows = kBlock;
   if (I.precision == SHELL_FP64)
     for (I.chunk_rows = 32; I.chunk_rows < kBlock && nv > 152 * I.chunk_rows;) I.chunk_rows *= 2;
