@@ -232,6 +232,17 @@ void destroy_graph(shell_batch *b) {
 // The step kernel's variant with the Newton tangent also carries the projection of per-component constraints.
 static bool uses_nt_variant(const Inst &I) { return (I.nl_newton && I.nl_max > 1) || I.fix != nullptr; }
 
+// Most CTAs an instance is given for its row blocks. A small FP64 instance has several (of 32 rows), but an iteration of it on
+// one CTA takes no longer than the barriers of a team: up to 128 vertices, and up to 64 with Newton iterations, whose
+// products are longer, it keeps one. Two steps from a given state of plates in FP64, team -> one CTA, alone / 24 in a batch:
+//   linearised  64 vertices 0.90 -> 0.66 / 0.97 -> 0.74 ms, 121 vertices 1.30 -> 0.95 / 1.37 -> 1.23 (240: 1.95 -> 1.60 / 2.07 -> 2.45)
+//   4 chord iterations  64: 2.59 -> 1.89 / 2.76 -> 2.09, 121: 3.73 -> 2.74 / 3.86 -> 3.45 (240: 5.67 -> 4.43 / 5.67 -> 6.90)
+//   Newton iterations   64: 11.9 -> 10.1 / 12.1 -> 11.9, 121: 17.4 -> 16.8 / 17.6 -> 26.3
+int most_ctas(const Inst &I) {
+  if (I.precision == SHELL_FP64 && I.nv <= (I.nl_newton && I.nl_max > 1 ? 64 : 128)) return 1;
+  return std::max(1, I.n_chunks);
+}
+
 // Build the force tile lists and the persistent-solve schedule for the resident instances.
 int rebuild_tables(shell_batch *b) {
   destroy_graph(b);
@@ -286,7 +297,7 @@ int rebuild_tables(shell_batch *b) {
   // the model's factor for the team it ran with) once the instance has run, else rows x iterations.
   constexpr double kBeta = 0.04;
   const double beta = kBeta * b->share_scale;
-  auto cmax = [&](int k) { return std::max(1, b->slots[b->active[k]]->h.n_chunks); };
+  auto cmax = [&](int k) { return most_ctas(b->slots[b->active[k]]->h); };
   auto factor = [&](int k, int c) {
     const double B = cmax(k);
     return std::ceil(B / c) / B * (1.0 + beta * (c - 1));
@@ -1549,7 +1560,7 @@ int shell_step_noalloc(shell_handle *h, int32_t n_steps, shell_step_stats *stats
   if (h->batch) return SHELL_ERR_BUSY;
   const bool newton = uses_nt_variant(h->h);
   const int prec = newton ? 3 : (h->h.precision == SHELL_FP64 ? 1 : 2);
-  int team = std::max(1, std::min(num_sms() * blocks_per_sm_cached(prec, prec == 2 ? 3 : 2), h->h.n_chunks));
+  int team = std::min(num_sms() * blocks_per_sm_cached(prec, prec == 2 ? 3 : 2), most_ctas(h->h));
   if (team > static_max_ctas()) return SHELL_ERR_STATIC_LIMIT;
   const InstStatus before = h->last_status;
   InstStatus after{};

@@ -38,3 +38,33 @@ def test_the_autotuner_tries_three_occupancies_in_fp32():
     assert all(ms > 0.0 for ms in info["trial_ms"][:9])
     assert info["ctas_per_sm"] in (2, 3, 4)
     gb.shell_batch_destroy(b)
+
+
+# 64, 72, 128 and 132 vertices; a narrow band (129 vertices) is one row block for the direct Newton solve in any case
+@pytest.mark.parametrize("nx,ny,newton,one", [(7, 7, True, True), (7, 8, True, False), (15, 7, False, True),
+                                              (11, 10, False, False), (42, 2, False, True)])
+def test_small_fp64_instances_take_one_cta(nx, ny, newton, one):
+    sc = sg.cylinder_panel(nx, "FS", ny=ny)
+
+    def make():
+        h = gb.create_from_scenario(sc, precision="fp64", pcg_rtol=1e-8)
+        if newton:
+            gb.shell_set_nonlinear(h, 3, 0.0)
+            gb.shell_set_newton(h, True)
+        return h
+
+    states = []
+    for batch in (1, 3):
+        hs = [make() for _ in range(batch)]
+        b = gb.shell_batch_create(1 << 40)
+        slots = [gb.shell_batch_admit(b, h) for h in hs]
+        for _ in range(2):
+            rc, stats = gb.shell_batch_step(b, 1)
+            assert rc == 0 and all((stats[k]["team_ctas"] == 1) == one for k in slots)
+        states.append(gb.shell_batch_get_states(b)[0][:sc.n_verts])
+        gb.shell_batch_destroy(b)
+    h = make()
+    st = gb.shell_step_noalloc(h, 2)
+    assert (st["team_ctas"] == 1) == one
+    states.append(gb.shell_get_state(h)[0])
+    assert (states[0] == states[1]).all() and (states[0] == states[2]).all()
