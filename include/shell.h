@@ -137,9 +137,9 @@ typedef struct shell_options {
                             * round also stops once its residual is 0.7 refine_rtol ||b||, with a dense inverse
                             * 0.07 refine_rtol ||b||) */
   double refine_rtol;      /* FP32_REFINE: stop when the FP64 residual ||b - A v|| <= refine_rtol ||b|| (a dense
-                            * inverse takes one further round in a linearised step, if refine_max allows it, where a
-                            * round ends above 0.07 of that: its rounding errors are smooth, and weigh more in the
-                            * result) */
+                            * inverse takes one further round, if refine_max allows it and the solve is not a later
+                            * Newton iteration's, where a round ends above 0.07 of that: its rounding errors are
+                            * smooth, and weigh more in the result) */
   int32_t pcg_max_it;      /* iteration cap per solve (per inner solve in FP32_REFINE) */
   int32_t refine_max;      /* FP32_REFINE: cap on refinement rounds */
   void *cuda_stream;       /* cudaStream_t, or NULL */

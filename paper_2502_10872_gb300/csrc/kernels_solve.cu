@@ -2225,8 +2225,9 @@ __device__ bool solve_fp32r(const Inst &I, Team &tm) {
     // A dense inverse as the preconditioner: what a round leaves is the rounding of the FP32 matrix and its inverse, which
     // lies in the smooth modes, where a residual stands for the most error (a multigrid round leaves some of every mode).
     // A first round that ends just under the target is up to 5 times as far off as a multigrid solve, so one further round
-    // is taken where a round ends above 0.07 of the target (not more than one: FP64 rounding may not allow it; none in
-    // chord and Newton iterations, where the next iteration starts from the true residual). 289-vertex
+    // is taken where a round ends above 0.07 of the target (not more than one: FP64 rounding may not allow it; not in Newton
+    // iterations, which remove what the solve before left, as chord iterations do not in modes that the constant matrix
+    // overestimates; not where the target is the nonlinear iteration's). 289-vertex
     // plate, six states, largest error of the displacement and time of a call: 6.7e-9 with the cycle (520 us), 3.3e-8
     // ending at the target (150 us), 2.1e-11 with the further round (177 us).
     bool met = false;
@@ -2252,7 +2253,8 @@ __device__ bool solve_fp32r(const Inst &I, Team &tm) {
       }
       if (writer) rel = sqrt(r2 / ref);
       if (r2 <= tol_ref2) {
-        if (I.amg_levels != 1 || I.nl_max > 1 || rounds == 0 || r2 <= 0.005 * tol_ref2 || met || rounds >= I.refine_max) break;
+        if (I.amg_levels != 1 || rounds == 0 || r2 <= 0.005 * tol_ref2 || met || rounds >= I.refine_max) break;
+        if (k > 0 && (I.nl_newton || tol_ref2 > I.refine_rtol * I.refine_rtol * ref)) break;
         met = true;
       }
       if (rounds >= I.refine_max) {
