@@ -74,12 +74,13 @@ class Server:
     """Admit requests into one batch by an HBM budget and step them together."""
 
     # Launch shape of the batch's step kernel (CTAs per SM, CTA-share scale, clusters), measured on the
-    # serving mix (1k-250k-vertex requests): the most CTAs per SM (5 asked for; the library's largest variant now
-    # holds 4) with a small share scale, so that the largest resident requests get large teams. Serving, 10 s on one box: the library's default (3 CTAs per
-    # SM, share 1) 134.8 M vertex-steps/s; (5, 2.0), the shape the autotuner picks for batches of instances
-    # of at most 66 row blocks, 51.8-56.3 M; (5, 1.0) 131.1 M; (5, 0.5) 186.3 M; (5, 0.25) 203.7-205.4 M;
-    # (5, 0.125) 211.6 M; (5, 0.0625) 208.8 M. None keeps the library's default.
-    DEFAULT_LAUNCH = (5, 0.125, False)
+    # serving mix (1k-250k-vertex requests): the most CTAs per SM with a small share scale, so that the
+    # largest resident requests get large teams. Measured while the largest variant held 5 CTAs per SM (4 since),
+    # serving, 10 s on one box: the library's default (3 CTAs per SM, share 1) 134.8 M vertex-steps/s; (5, 2.0), the shape
+    # the autotuner picks for batches of instances of at most 66 row blocks, 51.8-56.3 M; (5, 1.0) 131.1 M; (5, 0.5)
+    # 186.3 M; (5, 0.25) 203.7-205.4 M; (5, 0.125) 211.6 M; (5, 0.0625) 208.8 M. Now, with 4: 220.7-221.5 M, where the code
+    # with 5 gave 198.5-206.7 M on the same box. None keeps the library's default.
+    DEFAULT_LAUNCH = (4, 0.125, False)
 
     def __init__(self, budget_bytes: int, precision: str = "fp32_refine", keep_states: bool = False,
                  create_kw: Optional[dict] = None, clock: Callable[[], float] = time.perf_counter,
